@@ -145,7 +145,7 @@ static akra_status batch_reserve(akra_batch b)
         akra_plan p = b->plans[i];
         const int R = b->R[i];
         const LegShape s64 = leg_shape(p, AKRA_F64, R);
-        const size_t nch64 = legendre_chunks(p->n_active_units, s64);
+        const size_t nch64 = legendre_chunks(p, p->d_active_units, p->n_active_units, s64);
         const size_t part = std::max((size_t)b->nch[i] * R * p->ntri * 4 * sizeof(float),
                                      nch64 * R * p->ntri * 4 * sizeof(double));
         AKRA_TRY(ws_reserve(p, p->phi, (size_t)R * p->nring * (2 * (size_t)p->lmax + 1) * sizeof(double2)));

@@ -89,6 +89,7 @@ __device__ __forceinline__ long long dbg_index(long long i, long long bound, int
 #endif
 akra_status debug_collect_legendre(DebugRecord *acc);
 akra_status debug_collect_legendre_tc(DebugRecord *acc);
+akra_status debug_collect_legendre_blk(DebugRecord *acc);
 akra_status debug_collect_batch(DebugRecord *acc);
 akra_status debug_collect_ringfft(DebugRecord *acc);
 akra_status debug_collect_ringfft32(DebugRecord *acc);
@@ -176,9 +177,30 @@ struct LegShape {
     int TC = 0;            // FP32 synthesis on the tensor core with RHS groups of TC (4, 8, 16,
                            // 32); 0: CUDA-core synthesis of shape (P, RG)
     int RGA = 0;           // RHS per block of the adjoint (0: same as RG)
+    int BS = 0, BA = 0;    // FP32 synthesis / adjoint by 16-step block jumps (akra_legendre_blk.cuh)
     int adjP() const { return PA > 0 ? PA : P; }
     int adjRG() const { return RGA > 0 ? RGA : RG; }
 };
+
+// chunk of 256 rings of the block-jump Legendre kernels (akra_legendre_blk.cuh)
+struct BlkChunk {
+    float node[16];        // interpolation nodes in x = cos θ
+    float zmax;            // largest |x| of the chunk's interval
+    float pad[3];
+};
+
+// the rings (more than 0.1 rad from the poles) those kernels transform, in latitude order, with their
+// chunks and interpolation tables; npolar: ring pairs of the list's unit list left to the other kernels
+struct BlkTables {
+    int *rows = nullptr;
+    BlkChunk *info = nullptr;
+    uint4 *vtab = nullptr;
+    int nrows = 0, nchunks = 0, npolar = 0;
+    size_t cap_rows = 0;
+};
+
+// smallest band limit at which the block-jump kernels run (their smallest measured gain: 64 / 128)
+constexpr int kBlkMinLmax = 128;
 
 // arguments of one Legendre kernel instance (one plan; the batched launches hold an array)
 template <typename T>
@@ -206,6 +228,11 @@ struct LegArgs {
     const long long *tc_tilebase;
     int tc_groups;
     long long tc_tiles;
+    // block-jump kernels: ring rows, chunks and interpolation tables
+    const int *blk_rows;
+    const BlkChunk *blk_info;
+    const uint4 *blk_vtab;
+    int blk_nrows, blk_chunks;
 };
 
 // arguments of one FP32 ring-FFT instance
@@ -311,7 +338,11 @@ struct akra_plan_s {
     int *d_active_units = nullptr;           // units with an active ring
     int n_active_units = 0;
     int one_side = 0;                        // every active unit needs only its north (1) / south (2) ring
+    bool mostly_one_ring = false;            // at least half of the FP32 Legendre steps are on active units
+                                             // that need one ring only
     unsigned char *d_ring_active = nullptr;  // [nring] flag
+
+    akra::BlkTables blk_all, blk_act;        // block-jump Legendre tables: all rings, active rings
 
     // workspaces (grown on demand)
     akra::Workspace phi, partial, cg, red;
@@ -355,12 +386,23 @@ akra_status legendre_tc_bstage(int tcg, const LegArgs<float> &a, cudaStream_t st
 // persistent tensor-core synthesis over a work list of (instance, m, 128-pair chunk, RHS group)
 akra_status legendre_synth_tc_queue(int tcg, const LegArgs<float> *insts, const int4 *items, int nitems,
                                     int *counter, cudaStream_t st);
+// block-jump Legendre kernels (akra_legendre_blk.cu); rows: the ring rows of the list, ascending, and
+// npolar how many of its ring pairs lie within 0.1 rad of a pole
+akra_status blk_tables_build(akra_plan p, BlkTables &t, const std::vector<int> &rows, int npolar, cudaStream_t st);
+void blk_tables_free(BlkTables &t);
+akra_status legendre_blk_prepare();
+akra_status legendre_synth_blk(akra_plan p, LegMode mode, const void *alm, void *phi, int R, const int *units,
+                               cudaStream_t st);
+akra_status legendre_adjoint_blk(akra_plan p, const void *phi, void *partial, int R, const int *units, int nchunks,
+                                 cudaStream_t st);
+bool blk_pays(akra_plan p, const int *units, bool adjoint);
+inline const BlkTables &blk_tables(akra_plan p, const int *units) { return units == p->d_all_units ? p->blk_all : p->blk_act; }
 // reads and clears the plan's kernel-wait error flag (blocking): ECUDA if a bounded wait ran out
 akra_status tc_error_check(akra_plan p);
 
 
 LegShape leg_shape(akra_plan p, akra_prec prec, int R);
-int legendre_chunks(int nunits, const LegShape &s);
+int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s);
 void cg_release_graphs(akra_plan p);   // akra_cg.cu
 akra_status metric_inverse(akra_plan p, bool dbl, const void *in, void *out, int R, cudaStream_t st);
 

@@ -111,6 +111,12 @@ LegArgs<T> leg_args(akra_plan p, const LegShape &s, LegMode mode, const int *uni
     a.tc_tilebase = p->d_tc_tilebase;
     a.tc_groups = s.TC > 0 ? (R + s.TC - 1) / s.TC : 0;
     a.tc_tiles = p->tc_tiles;
+    const BlkTables &bt = blk_tables(p, units);
+    a.blk_rows = bt.rows;
+    a.blk_info = bt.info;
+    a.blk_vtab = bt.vtab;
+    a.blk_nrows = bt.nrows;
+    a.blk_chunks = bt.nchunks;
     return a;
 }
 
@@ -137,14 +143,37 @@ static int launch_adjoint(akra_plan p, const void *phi, void *partial, int R, co
     return a.nchunks;
 }
 
+// Whether the block-jump kernels take a list's ring pairs (FP32, unless the plan's shape rules them out).
+// They treat every ring by itself, the direct kernels share a pair's recurrence between its two rings, so
+// the line lies where most of the work is on pairs that need one ring.  One RHS, direct -> block-jump:
+// footprints of one hemisphere at (Nside, lmax) = (64, 128) synthesis 13.6 -> 10.9 us, adjoint 23.2 -> 14.3;
+// (512, 1024) 181 -> 125, 311 -> 223; (2048, 4096) 8.19 -> 4.16 ms, 10.31 -> 8.84 ms.  Full sky, whole
+// transforms: (1024, 2048) 2.08 -> 2.35 ms, 3.83 -> 4.66; (2048, 4096) 13.7 -> 12.1 ms, 19.7 -> 24.9: only
+// the synthesis, and only from lmax 4096 on.
+bool blk_pays(akra_plan p, const int *units, bool adjoint)
+{
+    if (p->lmax < kBlkMinLmax) return false;
+    if (units != p->d_all_units && p->mostly_one_ring) return true;
+    return !adjoint && p->lmax >= 4096;
+}
+
 // shape dispatch: (P, RG) combinations compiled for each precision, NT = 128
 template <typename T>
 akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const void *alm,
                            void *phi, int R, const int *units, int nunits, cudaStream_t st)
 {
     if (nunits <= 0) return AKRA_OK;
-    if constexpr (std::is_same<T, float>::value)
+    if constexpr (std::is_same<T, float>::value) {
         if (s.TC > 0) return legendre_synth_tc(p, s.TC, mode, alm, phi, R, units, nunits, st);
+        if (s.BS && blk_pays(p, units, false)) {
+            // the polar ring pairs (the first of the list) keep the difference-form kernels
+            const int npolar = blk_tables(p, units).npolar;
+            LegShape sp = s;
+            sp.BS = 0;
+            AKRA_TRY(legendre_synth<T>(p, sp, mode, alm, phi, R, units, npolar, st));
+            return legendre_synth_blk(p, mode, alm, phi, R, units, st);
+        }
+    }
 #define AKRA_S(PP, RR)                                                                      \
     if (s.P == PP && s.RG == RR) {                                                          \
         launch_synth<T, PP, RR, 128>(p, mode, alm, phi, R, units, nunits, st);              \
@@ -167,6 +196,19 @@ akra_status legendre_adjoint(akra_plan p, const LegShape &s, const void *phi, vo
     *nchunks_out = 0;
     if (nunits <= 0) return AKRA_OK;
     const int pa = s.adjP();
+    if constexpr (std::is_same<T, float>::value) {
+        if (s.BA && blk_pays(p, units, true)) {
+            // chunks of the block-jump kernel first, then those of the polar ring pairs (the first of the list)
+            const BlkTables &t = blk_tables(p, units);
+            LegShape sp = s;
+            sp.BA = 0;
+            int np = 0;
+            AKRA_TRY(legendre_adjoint<T>(p, sp, phi, (T *)partial + (size_t)t.nchunks * R * p->ntri * 4, R, units,
+                                         t.npolar, &np, st));
+            *nchunks_out = t.nchunks + np;
+            return legendre_adjoint_blk(p, phi, partial, R, units, *nchunks_out, st);
+        }
+    }
     {
         // the active ring pairs of a one-hemisphere footprint all need the same single ring: the
         // kernel compiled for that form alone (fewer registers); FP32 at 3-8 ring pairs per
@@ -214,9 +256,13 @@ akra_status adjoint_epilogue(akra_plan p, LegMode mode, const void *partial, int
 }
 
 // chunks of the adjoint (its partial sums are laid out per chunk)
-int legendre_chunks(int nunits, const LegShape &s)
+int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s)
 {
     const int per = s.NT * s.adjP();
+    if (s.BA && nunits > 0 && blk_pays(p, units, true)) {
+        const BlkTables &t = blk_tables(p, units);
+        return t.nchunks + (t.npolar + per - 1) / per;
+    }
     return (nunits + per - 1) / per;
 }
 

@@ -459,9 +459,9 @@ LegShape leg_shape(akra_plan p, akra_prec prec, int R)
         if (R >= 2) return LegShape{1, 128, 2, 2, 0, 2};
         return LegShape{1, 128, 1, 4};
     }
-    if (R >= 4) return LegShape{1, 128, 4, 5, 0, 1};
-    if (R >= 2) return LegShape{1, 128, 2, 5, 0, 1};
-    return LegShape{1, 128, 1, 5};
+    LegShape s{1, 128, R >= 4 ? 4 : R >= 2 ? 2 : 1, 5, 0, 1};
+    s.BS = s.BA = 1;   // the block-jump kernels where they pay (blk_pays)
+    return s;
 }
 
 template <typename T> static akra_prec prec_of();
@@ -500,7 +500,7 @@ akra_status op_adjoint(akra_plan p, LegMode mode, const void *map, void *alm, bo
     const int *rings = act ? p->d_active_rings : p->d_all_rings;
     const int nrings = act ? p->n_active_rings : p->nring;
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
-    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(nunits, s) * R * p->ntri * 4 *
+    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(p, units, nunits, s) * R * p->ntri * 4 *
                                            sizeof(T)));
     AKRA_TRY(ring_fft<T>(p, FftMode::Adjoint, p->phi.ptr, map, nullptr, weighted, R, rings, nrings, st));
     int nch = 0;
@@ -514,7 +514,7 @@ akra_status op_H(akra_plan p, const void *x, void *y, int R, cudaStream_t st)
     if (is_flat(p)) return flat_op_H<T>(p, x, y, R, st);
     const LegShape s = leg_shape(p, prec_of<T>(), R);
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
-    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(p->n_active_units, s) * R *
+    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(p, p->d_active_units, p->n_active_units, s) * R *
                                            p->ntri * 4 * sizeof(T)));
     AKRA_TRY(legendre_synth<T>(p, s, LegMode::KS, x, p->phi.ptr, R, p->d_active_units,
                                p->n_active_units, st));
@@ -557,6 +557,31 @@ template <typename P> static akra_status dev_alloc(akra_plan p, P **ptr, size_t 
 }
 
 namespace akra { akra_status ring_fft_prepare(akra_plan p); }
+
+// the block-jump kernels' tables of a ring list (ascending): the rings more than 0.1 rad from the poles, and
+// the number of the list's ring pairs nearer than that
+static akra_status blk_build(akra_plan p, BlkTables &t, const std::vector<int> &rings, cudaStream_t st)
+{
+    const int N = p->nside;
+    auto polar = [&](int r) {   // as the kernels decide it: cos θ of the pair's north ring (k_geometry)
+        const long long i = std::min(r, 4 * N - 2 - r) + 1;
+        const double omz = i < N ? (double)(i * i) / (3.0 * (double)((long long)N * N)) : (double)(2 * i - N) / (3.0 * (double)N);
+        return 1.0 - omz >= kDiffX;
+    };
+    std::vector<int> rows;
+    std::vector<char> pair(p->nunit, 0);
+    int npolar = 0;
+    for (int r : rings) {
+        if (!polar(r)) {
+            rows.push_back(r);
+            continue;
+        }
+        char &seen = pair[std::min(r, 4 * N - 2 - r)];
+        npolar += !seen;
+        seen = 1;
+    }
+    return blk_tables_build(p, t, rows, npolar, st);
+}
 
 static akra_status plan_build(akra_plan p)
 {
@@ -639,6 +664,12 @@ static akra_status plan_build(akra_plan p)
     AKRA_TRY(ring_fft_prepare(p));
     AKRA_TRY(ring_fft32_build(p));
     AKRA_TRY(legendre_tc_prepare());
+    AKRA_TRY(legendre_blk_prepare());
+    {
+        std::vector<int> rings(p->nring);
+        for (int r = 0; r < p->nring; r++) rings[r] = r;
+        AKRA_TRY(blk_build(p, p->blk_all, rings, nullptr));
+    }
     {
         // 16-step l-tiles of every m (from l0 = max(m, 2)), the tensor-core synthesis' B operand grid
         std::vector<long long> tb(L + 1);
@@ -714,6 +745,8 @@ extern "C" void akra_plan_destroy(akra_plan p)
                     p->bpre.ptr, p->d_tc_tilebase};
     for (void *q : ptrs)
         if (q) cudaFree(q);
+    blk_tables_free(p->blk_all);
+    blk_tables_free(p->blk_act);
     if (p->stream) cudaStreamDestroy(p->stream);
     if (p->ev_a) cudaEventDestroy(p->ev_a);
     if (p->ev_b) cudaEventDestroy(p->ev_b);
@@ -732,6 +765,7 @@ extern "C" akra_status akra_debug_violations(long long *count, int *site, long l
     AKRA_CUDA_TRY(cudaDeviceSynchronize());
     AKRA_TRY(debug_collect_legendre(&acc));
     AKRA_TRY(debug_collect_legendre_tc(&acc));
+    AKRA_TRY(debug_collect_legendre_blk(&acc));
     AKRA_TRY(debug_collect_batch(&acc));
     AKRA_TRY(debug_collect_ringfft(&acc));
     AKRA_TRY(debug_collect_ringfft32(&acc));
@@ -864,6 +898,12 @@ extern "C" akra_status akra_plan_set_weights(akra_plan p, const double *d_ninv, 
         }
     }
     p->one_side = one > 0 ? one : 0;
+    unsigned long long steps_one = 0, steps_all = 0;
+    for (size_t k = 0; k < units.size(); k++) {
+        steps_all += p->steps32[units[k]];
+        if (one_ring[k]) steps_one += p->steps32[units[k]];
+    }
+    p->mostly_one_ring = steps_all > 0 && 2 * steps_one >= steps_all;
     AKRA_CUDA_TRY(cudaMemcpy(p->d_ring_active, active.data(), nr, cudaMemcpyHostToDevice));
     if (!rings.empty())
         AKRA_CUDA_TRY(cudaMemcpy(p->d_active_rings, rings.data(), sizeof(int) * rings.size(),
@@ -885,6 +925,8 @@ extern "C" akra_status akra_plan_set_weights(akra_plan p, const double *d_ninv, 
     AKRA_CUDA_TRY(cudaStreamSynchronize(st));
     p->has_weights = true;
     p->ws_gen++;   // captured CG iterations hold the previous active lists and λ_eff
+    AKRA_TRY(blk_build(p, p->blk_act, rings, st));
+    AKRA_CUDA_TRY(cudaStreamSynchronize(st));   // later calls may come on other streams
     return ring_fft32_order(p, rings, p->d_fft32_rings_act, &p->fft32_nsmall_act);
 }
 
@@ -990,9 +1032,16 @@ static akra_status tune_one(akra_plan p, akra_prec prec, int R, cudaStream_t st)
     const int *units = p->has_weights ? p->d_active_units : p->d_all_units;
     const int nunits = p->has_weights ? p->n_active_units : p->nunit;
     if (nunits == 0) return AKRA_OK;
+    // FP32: the block-jump kernels, tried first (equal times keep them)
+    if (std::is_same<T, float>::value && blk_pays(p, units, false)) {
+        LegShape c{1, 128, 1, 5, 0, 1};
+        c.BS = 1;
+        c.BA = blk_pays(p, units, true);
+        cands.insert(cands.begin(), c);
+    }
     size_t max_part = 0;
     for (auto &c : cands)
-        max_part = std::max(max_part, (size_t)legendre_chunks(nunits, c) * (size_t)R * (size_t)p->ntri * 4 * sizeof(T));
+        max_part = std::max(max_part, (size_t)legendre_chunks(p, units, nunits, c) * (size_t)R * (size_t)p->ntri * 4 * sizeof(T));
     AKRA_TRY(ws_reserve(p, p->phi, (size_t)R * p->nring * (2 * (size_t)p->lmax + 1) * sizeof(cx_t<T>)));
     AKRA_TRY(ws_reserve(p, p->partial, max_part));
     void *alm = nullptr;
@@ -1058,12 +1107,12 @@ static akra_status tune_one(akra_plan p, akra_prec prec, int R, cudaStream_t st)
         for (size_t k = 0; k < cands.size(); k++) {  // ... with a CUDA-core synthesis shape k
             if (ts[k] + ta[j] >= best) continue;
             best = ts[k] + ta[j];
-            pick = LegShape{cands[k].P, cands[k].NT, cands[k].RG, cands[j].P, 0, cands[j].RG};
+            pick = LegShape{cands[k].P, cands[k].NT, cands[k].RG, cands[j].adjP(), 0, cands[j].RG, cands[k].BS, cands[j].BA};
         }
         for (size_t q = 0; q < tcs.size(); q++) {    // ... or with the tensor-core synthesis
             if (ttc[q] + ta[j] >= best) continue;
             best = ttc[q] + ta[j];
-            pick = LegShape{cands[j].P, cands[j].NT, cands[j].RG, cands[j].P, tcs[q], cands[j].RG};
+            pick = LegShape{cands[j].P, cands[j].NT, cands[j].RG, cands[j].adjP(), tcs[q], cands[j].RG, 0, cands[j].BA};
         }
     }
     p->shapes[(long long)prec * 1000 + (R > 999 ? 999 : R)] = pick;
@@ -1129,6 +1178,7 @@ extern "C" akra_status akra_plan_set_adjoint_shape(akra_plan p, akra_prec prec, 
     LegShape s = leg_shape(p, prec, R);
     s.PA = PA;
     s.RGA = RGA;
+    s.BA = 0;
     p->shapes[(long long)prec * 1000 + (R > 999 ? 999 : R)] = s;
     p->ws_gen++;   // captured CG iterations used the previous shape
     return AKRA_OK;
@@ -1193,7 +1243,7 @@ static akra_status time_stages(akra_plan p, int R, int reps, cudaStream_t st, do
 {
     const akra_prec prec = prec_of<T>();
     const LegShape s = leg_shape(p, prec, R);
-    const int nch = legendre_chunks(p->n_active_units, s);
+    const int nch = legendre_chunks(p, p->d_active_units, p->n_active_units, s);
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
     AKRA_TRY(ws_reserve(p, p->partial, (size_t)nch * R * p->ntri * 4 * sizeof(T)));
     void *x = nullptr, *y = nullptr;

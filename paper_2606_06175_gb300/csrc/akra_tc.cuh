@@ -46,6 +46,28 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b
                  :: "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// kind::f16 operands (FP16 in, FP32 accumulator).  Core matrices are 8 x 16 bytes (8 FP16) as above.
+//   K-major: element (row, k) at (row / 8) sbo + (k / 8) lbo + (row % 8) 16 + (k % 8) 2
+//   MN-major (idesc_f16's ta / tb = 1): (row, k) at (row / 8) sbo + (k / 8) lbo + (k % 8) 16 + (row % 8) 2
+__device__ __forceinline__ uint64_t sdesc_f16(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
+           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
+}
+
+__host__ __device__ constexpr uint32_t idesc_f16(int m, int n, int ta, int tb)
+{
+    return (1u << 4) | ((uint32_t)ta << 15) | ((uint32_t)tb << 16) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(m >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                 :: "r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
 // arrive on the mbarrier once every MMA this thread issued so far has completed
 __device__ __forceinline__ void commit(uint64_t *mbar)
 {
@@ -56,6 +78,11 @@ __device__ __forceinline__ void commit(uint64_t *mbar)
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, int count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar)), "r"(count));
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(mbar)) : "memory");
 }
 
 // an mbarrier with no pending arrivals goes back to plain shared memory (before a re-init)
@@ -110,6 +137,24 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4])
     v[1] = __uint_as_float(r1);
     v[2] = __uint_as_float(r2);
     v[3] = __uint_as_float(r3);
+}
+
+// 16 consecutive TMEM columns of this warp's 32 lanes; tmem_wait_ld() before the values are used
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+{
+    uint32_t (&r)[16] = reinterpret_cast<uint32_t (&)[16]>(v);
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+}
+// the wait is tied to the loaded registers, so that no use of them moves above it
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                   "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+                 :: "memory");
 }
 
 // 16-byte asynchronous copy global -> shared (cp.async, L2 only); src_bytes = 0 zero-fills the
