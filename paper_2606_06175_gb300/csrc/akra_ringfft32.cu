@@ -166,13 +166,16 @@ akra_status ring_fft32(akra_plan p, FftMode mode, void *phi, const void *map_in,
                        bool weighted, int R, const int *rings, int nrings, cudaStream_t st)
 {
     if (nrings <= 0) return AKRA_OK;
-    // the plan's own ring lists go out in two launches by convolution length
+    // The plan's own ring lists go out in two launches by convolution length where a block of the larger
+    // length reserves so much shared memory that only one fits on an SM (Nside above 1024); below that a
+    // second launch only adds its latency (one H at Nside 32: 28.7 -> 16.0 us, 128: 29.3 -> 20.2, 256: 39 -> 35).
     const int *list = rings;
     int nsmall = 0;
-    if (p->fft32_msmall > 0 && rings == p->d_active_rings && nrings == p->n_active_rings) {
+    const bool split = (size_t)(f32_slots(p->fft32_mmax) + F32_NT) * sizeof(float2) > 100 * 1024;
+    if (split && p->fft32_msmall > 0 && rings == p->d_active_rings && nrings == p->n_active_rings) {
         list = p->d_fft32_rings_act;
         nsmall = p->fft32_nsmall_act;
-    } else if (p->fft32_msmall > 0 && rings == p->d_all_rings && nrings == p->nring) {
+    } else if (split && p->fft32_msmall > 0 && rings == p->d_all_rings && nrings == p->nring) {
         list = p->d_fft32_rings_all;
         nsmall = p->fft32_nsmall_all;
     }

@@ -213,7 +213,7 @@ __device__ void bluestein(float2 *x, int n, int M, int logM, const float2 *__res
     const int n2 = 2 * n;
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         if (j < n) {
-            const float2 c = tw_ring[(int)(((long long)j * j) % n2)];
+            const float2 c = tw_ring[(unsigned)(j * j) % (unsigned)n2];
             const float2 v = x[pd(j)];
             // forward: x conj(c);  backward: conj(x c) (conjugation trick)
             x[pd(j)] = S < 0 ? cmc(v, c) : make_float2(v.x * c.x - v.y * c.y, -(v.x * c.y + v.y * c.x));
@@ -228,7 +228,7 @@ __device__ void bluestein(float2 *x, int n, int M, int logM, const float2 *__res
     dit<+1>(x, M, logM, tw2);
     const float inv = 1.0f / (float)M;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const float2 c = tw_ring[(int)(((long long)k * k) % n2)];
+        const float2 c = tw_ring[(unsigned)(k * k) % (unsigned)n2];
         const float2 y = x[pd(k)];
         // forward: conj(c) y / M;  backward: c conj(y) / M
         const float2 r = S < 0 ? cmc(y, c) : cmc(c, y);
