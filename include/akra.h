@@ -374,8 +374,8 @@ akra_status akra_plan_set_shape(akra_plan plan, akra_prec prec, int R, int P, in
 /* The adjoint's own tile shape for (prec, R): ring pairs per thread PA and RHS per block RGA,
  * which may differ from the synthesis' RG (the synthesis amortises its recurrence over the RHS
  * of a block, the adjoint's per-step warp reduction grows with them).  akra_plan_set_shape sets
- * RGA = RG; akra_autotune picks synthesis and adjoint shapes independently; the defaults take
- * PA = 5, RGA = 1 (FP32) and PA = 2, RGA = 2 (FP64) for several RHS.  (PA, RGA) must be a
+ * RGA = RG; akra_autotune picks synthesis and adjoint shapes independently; the defaults grow
+ * with the work per SM (PA from 1 to 4, RGA 1 or 2).  (PA, RGA) must be a
  * compiled shape (list above).  Errors: EINVAL. */
 akra_status akra_plan_set_adjoint_shape(akra_plan plan, akra_prec prec, int R, int PA, int RGA);
 akra_status akra_plan_get_adjoint_shape(akra_plan plan, akra_prec prec, int R, int *PA, int *RGA);

@@ -450,16 +450,31 @@ LegShape leg_shape(akra_plan p, akra_prec prec, int R)
     const long long key = (long long)prec * 1000 + (R > 999 ? 999 : R);
     auto it = p->shapes.find(key);
     if (it != p->shapes.end()) return it->second;
-    // defaults (measured on the DES-like footprint at Nside 1024-2048; akra_autotune refines):
-    // FP32 synthesis one ring pair per thread, with up to 4 RHS per block, and the paired adjoint
-    // at 5 pairs per thread, one RHS per block; FP64 synthesis up to 4 RHS per block, adjoint 2
-    // pairs per thread and 2 RHS per block (4 pairs, 1 RHS at R = 1)
+    // Defaults (akra_autotune refines), by W = ring-pair warps per SM at one pair per thread and one RHS per
+    // block, i.e. 2 Nside (lmax + 1) R / (32 · 152).  Several pairs or RHS per thread share work (recurrence,
+    // staged coefficients, the adjoint's warp reduction) but leave fewer warps: below W ~ 10 a block's own
+    // chain of steps is the time.  Measured in us (pairs, RHS per block), adjoint unless said:
+    //   FP64  W = 0.4 (32/64) (1,1) 39 (4,1) 86; W = 13 (128/256) (1,1) 301 (2,1) 289 (4,1) 447;
+    //         W = 54 (256/512) (2,1) 1083 (4,1) 1087; R = 4: W = 30 (2,1) 444 (2,2) 462, W = 54 (2,1) 665
+    //         (2,2) 539; synthesis R = 4: W = 14 (1,1) 97 (1,4) 167, W = 54 (1,2) 345 (1,4) 389, W = 216
+    //         (1,2) 2118 (1,4) 1817
+    //   FP32 (full sky; the block-jump kernels take the lists of blk_pays)  W = 10 (96/251) (1,1) 41 (2,1) 53
+    //         (5,1) 94; W = 121 (384/768) (2,1) 238 (3,1) 244 (5,1) 399; W = 403 (700/1400) (2,1) 1097 (3,1) 986
+    //         (5,1) 1541; W = 863 (1024/2048) (3,1) 2645 (4,1) 2567 (5,1) 3475; R = 4: W = 216 (2,1) 311 (2,2)
+    //         274 (5,1) 533
+    const double W = 2.0 * p->nside * (p->lmax + 1.0) * R / (32.0 * 152.0);
     if (prec == AKRA_F64) {
-        if (R >= 4) return LegShape{1, 128, 4, 2, 0, 2};
-        if (R >= 2) return LegShape{1, 128, 2, 2, 0, 2};
-        return LegShape{1, 128, 1, 4};
+        LegShape s{1, 128, R >= 4 && W >= 100 ? 4 : R >= 2 && W >= 20 ? 2 : 1};
+        s.PA = W < 8 ? 1 : W < 40 || R >= 2 ? 2 : 4;
+        s.RGA = W >= 40 && R >= 2 ? 2 : 1;
+        return s;
     }
-    LegShape s{1, 128, R >= 4 ? 4 : R >= 2 ? 2 : 1, 5, 0, 1};
+    LegShape s{1, 128, R >= 4 ? 4 : R >= 2 ? 2 : 1};
+    if (R >= 2 && W >= 40 && W < 1500) s.PA = s.RGA = 2;
+    else {
+        s.PA = W < 16 ? 1 : W < 150 ? 2 : W < 600 ? 3 : 4;
+        s.RGA = 1;
+    }
     s.BS = s.BA = 1;   // the block-jump kernels where they pay (blk_pays)
     return s;
 }
