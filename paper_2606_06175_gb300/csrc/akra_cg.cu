@@ -38,20 +38,31 @@ __device__ __forceinline__ double wdot<float>(bool m0, float2 a, float2 b)
     return (double)(m0 ? a.x * b.x : 2.f * fmaf(a.x, b.x, a.y * b.y));
 }
 
+// sum of one double per thread over the block, in thread 0 (fixed order: lanes, then warps)
+__device__ __forceinline__ double block_sum(double v, double *sh)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        v = threadIdx.x < RED_NT / 32 ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int off = RED_NT / 64; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    }
+    return v;
+}
+
 // block-reduce one double per slot into scratch[k * RED_NB + blockIdx.x]; returns true on the
-// last block to finish (which may then read every partial)
+// last block to finish (which may then read every partial).  The sums go through shuffles, two barriers a
+// slot: in solves of small plans these kernels are a chain of latencies, not of bytes.
 __device__ bool block_partials(double *vals, int nslots, double *scratch, CgCtl *ctl)
 {
-    __shared__ double sh[RED_NT];
+    __shared__ double sh[RED_NT / 32];
     __shared__ bool last;
     for (int r = 0; r < nslots; r++) {
-        sh[threadIdx.x] = vals[r];
-        __syncthreads();
-        for (int off = RED_NT / 2; off > 0; off >>= 1) {
-            if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) scratch[(size_t)r * RED_NB + blockIdx.x] = sh[0];
+        const double s = block_sum(vals[r], sh);
+        if (threadIdx.x == 0) scratch[(size_t)r * RED_NB + blockIdx.x] = s;
         __syncthreads();
     }
     __threadfence();
@@ -64,19 +75,21 @@ __device__ bool block_partials(double *vals, int nslots, double *scratch, CgCtl 
 // partials are read past L1, they were written by other blocks), into tot[0..nslots)
 __device__ void block_totals(const double *scratch, int nslots, double *tot)
 {
-    __shared__ double sh[RED_NT];
+    __shared__ double sh[RED_NT / 32];
     for (int r = 0; r < nslots; r++) {
         double s = 0;
-        for (int b = threadIdx.x; b < RED_NB; b += RED_NT) s += __ldcg(scratch + (size_t)r * RED_NB + b);
-        sh[threadIdx.x] = s;
-        __syncthreads();
-        for (int off = RED_NT / 2; off > 0; off >>= 1) {
-            if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) tot[r] = sh[0];
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += RED_NT) s += __ldcg(scratch + (size_t)r * RED_NB + b);
+        s = block_sum(s, sh);
+        if (threadIdx.x == 0) tot[r] = s;
         __syncthreads();
     }
+}
+
+// blocks of the vector kernels: no more than the vectors have work for (one element per thread and field)
+static int red_blocks(akra_plan p)
+{
+    const long long n = (p->ntri + RED_NT - 1) / RED_NT;
+    return (int)(n < 1 ? 1 : n < RED_NB ? n : RED_NB);
 }
 
 constexpr int kMaxRhsLocal = 64;
@@ -197,6 +210,7 @@ k_cg_update_xr(int L, long long ntri, const cx_t<T> *p, const cx_t<T> *q, cx_t<T
 {
     if (ctl->all_done) return;
     const int R = ctl->R;
+    const int ns = pw ? 2 : 1;   // sums per RHS: <r, r>, and <r, P r> where P is not a scalar
     double acc[2 * kMaxRhsLocal];
     for (int r = 0; r < R; r++) {
         double a = 0, az = 0;
@@ -216,21 +230,21 @@ k_cg_update_xr(int L, long long ntri, const cx_t<T> *p, const cx_t<T> *q, cx_t<T
                 if (pw) az += (double)pw[j] * d;
             }
         }
-        acc[2 * r] = a;
-        acc[2 * r + 1] = az;
+        acc[ns * r] = a;
+        if (pw) acc[ns * r + 1] = az;
     }
-    if (block_partials(acc, 2 * R, scratch, ctl)) {
+    if (block_partials(acc, ns * R, scratch, ctl)) {
         __shared__ double tot[2 * kMaxRhsLocal];
-        block_totals(scratch, 2 * R, tot);
+        block_totals(scratch, ns * R, tot);
         const double P = ctl->precond;
         for (int r = threadIdx.x; r < R; r += RED_NT) {
             CgState s = st[r];
             if (s.done) continue;
-            const double rr = tot[2 * r];
+            const double rr = tot[ns * r];
             s.rr = rr;
             s.iters += 1;
             s.relres = sqrt(rr / s.bnorm2);
-            const double rz_new = pw ? tot[2 * r + 1] : P * rr;
+            const double rz_new = pw ? tot[ns * r + 1] : P * rr;
             s.beta = rz_new / s.rz;
             s.rz = rz_new;
             if (!isfinite(rr)) {
@@ -526,7 +540,7 @@ static akra_status true_residual(akra_plan p, int R, CgBufs &b, const void *bv, 
 {
     cudaStream_t cs = p->stream;
     AKRA_TRY(op_H<T>(p, xv, tmp, R, cs));
-    k_residual<T><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const cx_t<T> *)bv,
+    k_residual<T><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const cx_t<T> *)bv,
                                              (const cx_t<T> *)tmp, (cx_t<T> *)rout, b.res,
                                              b.ctl[PrecIdx<T>::v], b.scratch);
     AKRA_CUDA_TRY(cudaGetLastError());
@@ -596,7 +610,7 @@ static akra_status solve_b(akra_plan p, akra_prec prec, const void *bsrc, void *
         AKRA_CUDA_TRY(cudaMemsetAsync(x64, 0, V64, cs));
         AKRA_CUDA_TRY(cudaMemsetAsync(t64, 0, V64, cs));
         // r = b - H·0 = b  (residual kernel with h = 0 gives ||r||, ||b||)
-        k_residual<double><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const double2 *)b64,
+        k_residual<double><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const double2 *)b64,
                                                      (const double2 *)t64, (double2 *)r64, b.res,
                                                      b.ctl[0], b.scratch);
         AKRA_CUDA_TRY(cudaGetLastError());
@@ -686,7 +700,7 @@ akra_status cg_launch_init(akra_plan p, int R, CgBufs &b, double tol, int maxite
     hctl.maxiter = maxiter;
     // pageable-to-device copies are staged and ordered on the stream
     AKRA_CUDA_TRY(cudaMemcpyAsync(ctl, &hctl, sizeof(CgCtl), cudaMemcpyHostToDevice, cs));
-    k_cg_init<T><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[0], (cx_t<T> *)v[1],
+    k_cg_init<T><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[0], (cx_t<T> *)v[1],
                                             (cx_t<T> *)v[2], (cx_t<T> *)v[3], st, ctl, b.scratch, tol,
                                             maxiter, pw_ptr<T>(p));
     AKRA_CUDA_TRY(cudaGetLastError());
@@ -700,12 +714,12 @@ akra_status cg_launch_tail(akra_plan p, CgBufs &b, cudaStream_t cs)
     void **v = vecs<T>(b);
     CgState *st = b.st[PrecIdx<T>::v];
     CgCtl *ctl = b.ctl[PrecIdx<T>::v];
-    k_cg_dot_pq<T><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[3],
+    k_cg_dot_pq<T><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[3],
                                               (const cx_t<T> *)v[4], st, ctl, b.scratch);
-    k_cg_update_xr<T><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[3],
+    k_cg_update_xr<T><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, (const cx_t<T> *)v[3],
                                                  (const cx_t<T> *)v[4], (cx_t<T> *)v[1],
                                                  (cx_t<T> *)v[2], st, ctl, b.scratch, pw_ptr<T>(p));
-    k_cg_update_p<T><<<RED_NB, RED_NT, 0, cs>>>(p->ntri, (const cx_t<T> *)v[2], (cx_t<T> *)v[3], st, ctl,
+    k_cg_update_p<T><<<red_blocks(p), RED_NT, 0, cs>>>(p->ntri, (const cx_t<T> *)v[2], (cx_t<T> *)v[3], st, ctl,
                                                 pw_ptr<T>(p));
     AKRA_CUDA_TRY(cudaGetLastError());
     return AKRA_OK;
@@ -714,7 +728,7 @@ akra_status cg_launch_tail(akra_plan p, CgBufs &b, cudaStream_t cs)
 akra_status launch_residual64(akra_plan p, int R, CgBufs &b, const void *bv, const void *hv, void *out,
                               cudaStream_t cs)
 {
-    k_residual<double><<<RED_NB, RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const double2 *)bv,
+    k_residual<double><<<red_blocks(p), RED_NT, 0, cs>>>(p->lmax, p->ntri, R, (const double2 *)bv,
                                                  (const double2 *)hv, (double2 *)out, b.res, b.ctl[0],
                                                  b.scratch);
     AKRA_CUDA_TRY(cudaGetLastError());
