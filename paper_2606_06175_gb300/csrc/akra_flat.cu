@@ -8,20 +8,29 @@
 //   H x   = conj(D) F (W F^-1 (D x)) + λ_eff x,   W = M N^-1 on the pixels,
 // the flat-sky Kaiser-Squires kernel (D(0) = 0) in place of D_l and the spin-2 SHTs.
 //
-// A 2D transform is a pass of row FFTs, a transpose, and a second pass of row FFTs; for H the
-// second and third passes (inverse along y, ×W, forward along y) are one kernel per row of the
-// transposed field, as the ring FFT fuses W between its two DFTs.  Row FFTs run in shared memory
-// (radix-4/2, decimation in frequency for the inverse, in time for the forward transform);
-// permutations are folded into the loads and stores.
+// A 2D transform is two passes of row FFTs; a pass writes its result transposed, so that the next one
+// reads rows again, and for H the second and third passes (inverse along y, ×W, forward along y) are one
+// kernel per row of the transposed field, as the ring FFT fuses W between its two DFTs.
+//
+// Row FFTs are radix-16 Stockham passes (plus one pass of radix 2, 4 or 8 where log2 n is no multiple of 4),
+// 16 elements of a row in each thread's registers: a row of 2048 crosses shared memory twice instead of the
+// six times of radix-4 passes, consecutive threads load consecutive twiddles, and the first pass reads and the
+// last writes global memory directly.  n is a template argument, which leaves one address and immediate
+// offsets per pass: with n at run time the index arithmetic was 35% of the issue slots and H took 129 us.
+// H at n = 2048, FP32: 95 us in three launches (0.2 GB through the L2), 247 us as five launches of radix-4
+// passes and transposes (0.34 GB); 512: 24 against 36; 8192: 1545 against 4429; 2048 FP64: 1.46 ms against 1.75.
+// FP32 is bound by issue and the L2 latency of the loads, which two blocks per SM cover in part; FP64 by the
+// FP64 pipe.
 #include "akra_internal.cuh"
 
 namespace akra {
 namespace flat {
 
-constexpr int NT = 512;            // threads per row-FFT block
-constexpr int kMaxN = 8192;        // largest grid side (FP64 rows: 139 KB of shared memory)
+constexpr int kMaxN = 8192;        // largest grid side
 
-__host__ __device__ constexpr int slots(int n) { return n + (n >> 4); }
+// a row's slots in shared memory: one of padding in 17, and 4 so that the rows of a transposed store are
+// read from different banks
+__host__ __device__ constexpr int slots(int n) { return n + (n >> 4) + 4; }
 __device__ __forceinline__ int pd(int i) { return i + (i >> 4); }   // bank-conflict padding
 
 // complex helpers on float2 / double2 (C)
@@ -35,88 +44,153 @@ template <int S, typename C> __device__ __forceinline__ C mul_si(C a)   // S i a
 {
     return S > 0 ? C{-a.y, a.x} : C{a.y, -a.x};
 }
-// e^{S 2πi t/len} from the table e^{-2πi u/n}
-template <int S, typename C>
-__device__ __forceinline__ C tw(const C *__restrict__ w, int t, int len, int n)
+
+// DFTs of sign S in registers, natural order in and out: v[r] <- Σ_q v[q] e^{S 2πi qr/N}
+template <int S, typename C> __device__ __forceinline__ void dft4(C &a, C &b, C &c, C &d)
 {
-    C v = w[t * (n / len)];
-    if (S > 0) v.y = -v.y;
-    return v;
+    const C s0 = cadd(a, c), d0 = csub(a, c), s1 = cadd(b, d), d1 = mul_si<S>(csub(b, d));
+    a = cadd(s0, s1);
+    b = cadd(d0, d1);
+    c = csub(s0, s1);
+    d = csub(d0, d1);
 }
 
-// in-place DIF, sign S: natural order in, bit-reversed out
-template <int S, typename T>
-__device__ void dif(cx_t<T> *x, int n, int logn, const cx_t<T> *__restrict__ w)
+// e^{S 2πi m/16}: cosines of 0, π/8, .. π/2 and symmetry (m a compile-time constant after unrolling)
+template <int S, typename T> __device__ __forceinline__ cx_t<T> root16(int m)
 {
-    int L = n;
-    if (logn & 1) {
-        const int h = n >> 1;
-        for (int i = threadIdx.x; i < h; i += NT) {
-            const cx_t<T> a = x[pd(i)], b = x[pd(i + h)];
-            x[pd(i)] = cadd(a, b);
-            x[pd(i + h)] = cmul(csub(a, b), tw<S>(w, i, n, n));
-        }
-        __syncthreads();
-        L = h;
-    }
-    for (; L >= 4; L >>= 2) {
-        const int q = L >> 2;
-        for (int b = threadIdx.x; b < (n >> 2); b += NT) {
-            const int blk = b / q, i = b - blk * q, t = blk * L + i;
-            const cx_t<T> a0 = x[pd(t)], a1 = x[pd(t + q)], a2 = x[pd(t + 2 * q)], a3 = x[pd(t + 3 * q)];
-            const cx_t<T> u0 = cadd(a0, a2), u1 = cadd(a1, a3), d0 = csub(a0, a2);
-            const cx_t<T> d1 = mul_si<S>(csub(a1, a3));
-            x[pd(t)] = cadd(u0, u1);
-            x[pd(t + q)] = cmul(csub(u0, u1), tw<S>(w, 2 * i, L, n));
-            x[pd(t + 2 * q)] = cmul(cadd(d0, d1), tw<S>(w, i, L, n));
-            x[pd(t + 3 * q)] = cmul(csub(d0, d1), tw<S>(w, 3 * i, L, n));
-        }
-        __syncthreads();
-    }
+    const T c[5] = {T(1), T(0.92387953251128675613), T(0.70710678118654752440), T(0.38268343236508977173), T(0)};
+    auto cs = [&](int k) { k &= 15; return k <= 4 ? c[k] : k <= 8 ? -c[8 - k] : k <= 12 ? -c[k - 8] : c[16 - k]; };
+    return cx_t<T>{cs(m), S > 0 ? cs(m + 12) : -cs(m + 12)};
 }
 
-// in-place DIT, sign S: bit-reversed order in, natural out
-template <int S, typename T>
-__device__ void dit(cx_t<T> *x, int n, int logn, const cx_t<T> *__restrict__ w)
+// R-point DFT of v[0..R) for R = 2, 4, 8, 16 as 4-point DFTs over the high digit, roots, and DFTs over the low one
+template <int S, typename T, int R> __device__ __forceinline__ void dft(cx_t<T> *v)
 {
-    const int Lmax = (logn & 1) ? (n >> 1) : n;
-    for (int L = 4; L <= Lmax; L <<= 2) {
-        const int q = L >> 2;
-        for (int b = threadIdx.x; b < (n >> 2); b += NT) {
-            const int blk = b / q, i = b - blk * q, t = blk * L + i;
-            const cx_t<T> p0 = x[pd(t)], p1 = x[pd(t + q)], p2 = x[pd(t + 2 * q)], p3 = x[pd(t + 3 * q)];
-            const cx_t<T> w1 = tw<S>(w, i, L, n), w2 = tw<S>(w, 2 * i, L, n);
-            cx_t<T> u = cmul(p1, w2);
-            const cx_t<T> u0 = cadd(p0, u), u1 = csub(p0, u);
-            u = cmul(p3, w2);
-            const cx_t<T> u2 = cadd(p2, u), u3 = csub(p2, u);
-            const cx_t<T> v2 = cmul(u2, w1), v3 = mul_si<S>(cmul(u3, w1));
-            x[pd(t)] = cadd(u0, v2);
-            x[pd(t + 2 * q)] = csub(u0, v2);
-            x[pd(t + q)] = cadd(u1, v3);
-            x[pd(t + 3 * q)] = csub(u1, v3);
+    using C = cx_t<T>;
+    if constexpr (R == 2) {
+        const C a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
+    } else if constexpr (R == 4) {
+        dft4<S>(v[0], v[1], v[2], v[3]);
+    } else {
+        constexpr int B = R / 4;   // q = B a + b, r = c + 4 d
+#pragma unroll
+        for (int b = 0; b < B; b++) {
+            dft4<S>(v[b], v[b + B], v[b + 2 * B], v[b + 3 * B]);   // over a: slot b + B c
+#pragma unroll
+            for (int c = 1; c < 4; c++)
+                if (b > 0) v[b + B * c] = cmul(v[b + B * c], root16<S, T>(b * c * (16 / R)));
         }
-        __syncthreads();
-    }
-    if (logn & 1) {
-        const int h = n >> 1;
-        for (int i = threadIdx.x; i < h; i += NT) {
-            const cx_t<T> a = x[pd(i)], b = cmul(x[pd(i + h)], tw<S>(w, i, n, n));
-            x[pd(i)] = cadd(a, b);
-            x[pd(i + h)] = csub(a, b);
+        C o[R];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            C w[B];
+#pragma unroll
+            for (int b = 0; b < B; b++) w[b] = v[B * c + b];
+            dft<S, T, B>(w);
+#pragma unroll
+            for (int d = 0; d < B; d++) o[c + 4 * d] = w[d];
         }
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; r++) v[r] = o[r];
     }
 }
 
-__device__ __forceinline__ int brev(int k, int logn) { return (int)(__brev((unsigned)k) >> (32 - logn)); }
-__device__ __forceinline__ int freq(int i, int n) { return i < n / 2 ? i : i - n; }
+// A row of N = 2^LOGN in N/16 threads: radix-16 passes and one of R0 = 2^(LOGN mod 4) where that is not 1.  Everything
+// but the thread's index is a compile-time constant, so that the accesses of a pass are one address and
+// immediate offsets.
+template <typename T, int LOGN>
+struct Row {
+    using C = cx_t<T>;
+    static constexpr int N = 1 << LOGN, TN = N / 16, R0 = 1 << (LOGN & 3);
+    static constexpr int R1 = R0 > 1 ? R0 : 16;   // first pass of the backward transform, last of the forward one
 
-// flat-sky Kaiser-Squires kernel at frequency indices (k1, k2)
+    // offset from t of the place of v[i] as the first pass of radix R reads it and the last one leaves it
+    template <int R> static __host__ __device__ constexpr int place(int i) { return (i / R) * TN + (i % R) * (16 / R) * TN; }
+
+    // slot of element i + off
+    static __device__ __forceinline__ int at(int i, int off)
+    {
+        return off % 16 == 0 ? pd(i) + off + off / 16 : pd(i + off);
+    }
+
+    // Stockham pass of radix R after passes of product Ns: butterflies j = t + u TN (u < 16/R), inputs
+    // x[j + q N/R] in v[u R + q], twiddled by e^{S 2πi qk/(Ns R)}, k = j mod Ns (table w[(q - 1) Ns + k],
+    // sign -), outputs x[(j - k) R + k + r Ns]
+    template <int S, int R, int Ns> static __device__ __forceinline__ void pass(C (&v)[16], int t, const C *__restrict__ w)
+    {
+#pragma unroll
+        for (int u = 0; u < 16 / R; u++) {
+            if (Ns > 1) {
+                const C *wk = w + ((t + u * TN) & (Ns - 1));
+#pragma unroll
+                for (int q = 1; q < R; q++) {
+                    C c = wk[(q - 1) * Ns];
+                    if (S > 0) c.y = -c.y;
+                    v[u * R + q] = cmul(v[u * R + q], c);
+                }
+            }
+            dft<S, T, R>(v + u * R);
+        }
+    }
+    // its outputs to the row's buffer; (k + r Ns) / 16 = r Ns / 16 for every pass
+    template <int R, int Ns> static __device__ __forceinline__ void put(C *buf, const C (&v)[16], int t)
+    {
+#pragma unroll
+        for (int u = 0; u < 16 / R; u++) {
+            const int k = (t + u * TN) & (Ns - 1);
+            const int o = Ns == 1 ? at(t * R, u * TN * R) : pd((t + u * TN - k) * R + k);
+#pragma unroll
+            for (int r = 0; r < R; r++) buf[o + r * Ns + (r * Ns >> 4)] = v[u * R + r];
+        }
+    }
+    // inputs of a pass of radix R
+    template <int R> static __device__ __forceinline__ void get(const C *buf, C (&v)[16], int t)
+    {
+#pragma unroll
+        for (int i = 0; i < 16; i++) v[i] = buf[at(t, place<R>(i))];
+    }
+
+    // radix-16 passes from Ns to the product M; then the buffer holds the inputs of a pass of radix R0, or v the row
+    template <int S, int Ns, int M> static __device__ __forceinline__ void passes16(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    {
+        if constexpr (Ns < M) {
+            pass<S, 16, Ns>(v, t, w);
+            if constexpr (Ns * 16 < N) {
+                __syncthreads();   // the buffer's last readers
+                put<16, Ns>(buf, v, t);
+                __syncthreads();
+                if constexpr (Ns * 16 < M) get<16>(buf, v, t);
+            }
+            passes16<S, Ns * 16, M>(v, buf, t, w + (Ns > 1 ? 15 * Ns : 0));
+        } else if constexpr (M < N) {
+            get<R0>(buf, v, t);
+            pass<S, R0, M>(v, t, w);
+        }
+    }
+    // Backward: R0, 16, 16, ..; forward: 16, 16, .., R0.  The backward transform ends and the forward one starts
+    // with the same radix-16 places, so ×W between them needs no exchange.
+    static __device__ __forceinline__ void backward(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    {
+        if constexpr (R0 > 1) {
+            pass<+1, R0, 1>(v, t, w);
+            put<R0, 1>(buf, v, t);
+            __syncthreads();
+            get<16>(buf, v, t);
+        }
+        passes16<+1, R0, N>(v, buf, t, w);
+    }
+    static __device__ __forceinline__ void forward(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    {
+        passes16<-1, 1, N / R0>(v, buf, t, w);
+    }
+};
+
+// flat-sky Kaiser-Squires kernel at frequencies (a, b)
 template <typename T>
-__device__ __forceinline__ cx_t<T> ks(int k1, int k2, int n)
+__device__ __forceinline__ cx_t<T> ks(T a, T b)
 {
-    const T a = (T)freq(k1, n), b = (T)freq(k2, n);
     const T q = a * a + b * b;
     if (q == T(0)) return cx_t<T>{0, 0};
     const T inv = T(1) / q;
@@ -125,71 +199,125 @@ __device__ __forceinline__ cx_t<T> ks(int k1, int k2, int n)
 
 template <typename T>
 struct Args {
-    int n, logn;
-    const cx_t<T> *w;        // twiddles e^{-2πi t/n}
+    bool tr;                 // the result goes to out[r][column][row]
+    const cx_t<T> *wb, *wf;  // twiddles of the backward and of the forward passes
     const cx_t<T> *in;       // [R][n][n]
-    cx_t<T> *out;            // [R][n][n] (may equal in)
+    cx_t<T> *out;            // [R][n][n]
     const T *Wt;             // middle pass: [n][n] weights, transposed, scaled by 1/n^2
     const cx_t<T> *xreg;     // mode 2: x for the λ_eff term (nullptr: none)
     T lam, scale;
     const int *skip;         // device flag: return at once if set
 };
 
-// One row of one RHS per block.  MODE
+// Up to 4096 a pass stores its rows transposed; rows of 8192, of which a block would hold too few for a
+// sector, are stored as they are and go through k_transpose.
+__host__ __device__ constexpr bool fused_transpose(int n) { return n <= 4096; }
+
+// Rows of a block.  A transposed store joins 32 bytes, a sector, from 4 FP32 rows: at n = 2048 H takes 95 us against
+// 100 with two, at 4096 (1024 threads) 361 against 425.  FP64 blocks are of 256 threads where that holds a row: at
+// 4096 one row takes 6.03 ms against 6.43 with two, the FP64 pipe being the bound.  Short rows fill 128 threads.
+template <typename T> __host__ __device__ constexpr int rows_per_block(int n)
+{
+    const int sector = 32 / (int)sizeof(cx_t<T>), threads = sizeof(T) == 8 ? 256 : fused_transpose(n) ? 1024 : 512;
+    const int most = threads * 16 / n < 1 ? 1 : threads * 16 / n, least = 128 * 16 / n < n ? 128 * 16 / n : n;
+    const int rows = sector < most ? sector : most;
+    return least > rows ? least : rows;
+}
+
+template <typename T> __host__ __device__ constexpr int row_threads(int n) { return rows_per_block<T>(n) * (n / 16); }
+
+// Registers: 64 a thread in FP32 (1024 threads per SM; 768 take 101 us for H at 2048, where 1024 take 95), 128 in FP64.
+template <typename T> constexpr int row_blocks(int n)
+{
+    return (sizeof(T) == 4 ? 1024 : 512) / (row_threads<T>(n) < 128 ? 128 : row_threads<T>(n));
+}
+
+// rows_per_block rows of one RHS per block, n/16 threads a row.  MODE
 //   0: ×D(k1 = column, k2 = row), inverse FFT along the row
 //   1: inverse FFT, ×Wt[row][y], forward FFT (the transposed middle of H)
 //   2: forward FFT, then ×conj(D(k1 = column, k2 = row)) × scale + λ x
 //   3: inverse FFT, × scale
 //   4: forward FFT
-template <typename T, int MODE>
-__global__ void __launch_bounds__(NT) k_rows(Args<T> a)
+template <typename T, int MODE, int LOGN>
+__global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << LOGN)) k_rows(Args<T> a)
 {
+    using C = cx_t<T>;
+    using F = Row<T, LOGN>;
+    constexpr int n = F::N, tn = F::TN, rpb = rows_per_block<T>(n);
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx_t<T> *buf = reinterpret_cast<cx_t<T> *>(smem_raw);
-    const int n = a.n, logn = a.logn, row = blockIdx.x;
-    const size_t base = ((size_t)blockIdx.y * n + row) * n;
-    const cx_t<T> *src = a.in + base;
-    cx_t<T> *dst = a.out + base;
-    constexpr bool fwd_first = MODE == 2 || MODE == 4;
-    for (int k = threadIdx.x; k < n; k += NT) {
-        cx_t<T> v = src[k];
-        if (MODE == 0) v = cmul(ks<T>(k, row, n), v);
-        buf[pd(fwd_first ? brev(k, logn) : k)] = v;   // DIT reads bit-reversed order
+    const int lt = threadIdx.x / tn, t = threadIdx.x % tn;
+    const int row = blockIdx.x * rpb + lt;
+    C *buf = reinterpret_cast<C *>(smem_raw) + lt * slots(n);
+    const size_t base = ((size_t)blockIdx.y * n + row) * n + t;
+    constexpr bool fwd_only = MODE == 2 || MODE == 4;
+    constexpr int RI = fwd_only ? 16 : F::R1;                          // first pass
+    constexpr int RO = MODE == 0 || MODE == 3 ? 16 : F::R1;            // last pass
+    const T ft = (T)t, fr = (T)(row < n / 2 ? row : row - n);          // frequencies; n/2 is a multiple of tn
+    auto fcol = [&](int off) { return ft + (T)(off < n / 2 ? off : off - n); };
+    C v[16];
+    const C *in = a.in + base;
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        const int off = F::template place<RI>(i);
+        v[i] = in[off];
+        if (MODE == 0) v[i] = cmul(ks<T>(fcol(off), fr), v[i]);
     }
-    __syncthreads();
-    if (fwd_first) {
-        dit<-1, T>(buf, n, logn, a.w);
-    } else {
-        dif<+1, T>(buf, n, logn, a.w);
-        if (MODE == 1) {
-            for (int k = threadIdx.x; k < n; k += NT) {
-                const T wy = a.Wt[(size_t)row * n + brev(k, logn)];
-                buf[pd(k)].x *= wy;
-                buf[pd(k)].y *= wy;
-            }
-            __syncthreads();
-            dit<-1, T>(buf, n, logn, a.w);
+    if (!fwd_only) F::backward(v, buf, t, a.wb);
+    if (MODE == 1) {
+        const T *wt = a.Wt + (size_t)row * n + t;
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            const T wy = wt[F::template place<16>(i)];
+            v[i].x *= wy;
+            v[i].y *= wy;
         }
     }
-    for (int k = threadIdx.x; k < n; k += NT) {
-        // after an inverse-only pass element k sits in bit-reversed slot brev(k)
-        cx_t<T> v = buf[pd((MODE == 0 || MODE == 3) ? brev(k, logn) : k)];
-        if (MODE == 2) {
-            const cx_t<T> d = ks<T>(k, row, n);
-            v = cmul(cx_t<T>{d.x, -d.y}, v);
-            v.x *= a.scale;
-            v.y *= a.scale;
+    if (fwd_only || MODE == 1) F::forward(v, buf, t, a.wf);
+    if (MODE == 3) {
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            v[i].x *= a.scale;
+            v[i].y *= a.scale;
+        }
+    }
+    if (MODE == 2) {
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            const int off = F::template place<RO>(i);
+            const C d = ks<T>(fcol(off), fr);
+            v[i] = cmul(C{d.x, -d.y}, v[i]);
+            v[i].x *= a.scale;
+            v[i].y *= a.scale;
             if (a.xreg) {
-                const cx_t<T> xr = a.xreg[base + k];
-                v.x = fma(a.lam, xr.x, v.x);
-                v.y = fma(a.lam, xr.y, v.y);
+                const C xr = a.xreg[base + off];
+                v[i].x = fma(a.lam, xr.x, v[i].x);
+                v[i].y = fma(a.lam, xr.y, v[i].y);
             }
-        } else if (MODE == 3) {
-            v.x *= a.scale;
-            v.y *= a.scale;
         }
-        dst[k] = v;
+    }
+    if (MODE == 2 || !a.tr) {
+        C *out = a.out + base;
+#pragma unroll
+        for (int i = 0; i < 16; i++) out[F::template place<RO>(i)] = v[i];
+    } else if constexpr (rpb * sizeof(C) >= 16) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 16; i++) buf[F::at(t, F::template place<RO>(i))] = v[i];
+        __syncthreads();
+        constexpr int RC = 16 / sizeof(C);   // rows in a 16-byte store
+        struct alignas(16) Chunk { C c[RC]; };
+        constexpr int nc = rpb / RC;         // stores side by side in a column
+        const int k = threadIdx.x / nc, r = (threadIdx.x % nc) * RC;
+        const C *src = reinterpret_cast<const C *>(smem_raw) + r * slots(n);
+        C *dst = a.out + ((size_t)blockIdx.y * n + k) * n + blockIdx.x * rpb + r;
+#pragma unroll
+        for (int i = 0; i < 16 / RC; i++) {
+            Chunk o;
+#pragma unroll
+            for (int q = 0; q < RC; q++) o.c[q] = src[q * slots(n) + F::at(k, i * tn * RC)];
+            *reinterpret_cast<Chunk *>(dst + (size_t)i * (tn * RC) * n) = o;
+        }
     }
 }
 
@@ -273,14 +401,16 @@ __global__ void k_weights(int n, const double *ninv, double *W64, float *W32, do
         for (int q = 0; q < 3; q++) atomicAdd(&stats[q], sh[q][0]);
 }
 
-__global__ void k_twiddles(int n, double2 *w64, float2 *w32)
+// twiddles of one pass: w[(q - 1) Ns + k] = e^{-2πi qk/(Ns R)}, 1 <= q < R, k < Ns
+__global__ void k_twiddles(int Ns, int R, double2 *w64, float2 *w32)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (R - 1) * Ns) {
+        const int q = 1 + i / Ns, k = i % Ns;
         double s, c;
-        sincospi(-2.0 * (double)t / (double)n, &s, &c);
-        w64[t] = make_double2(c, s);
-        w32[t] = make_float2((float)c, (float)s);
+        sincospi(-2.0 * (double)(q * k) / (double)(Ns * R), &s, &c);
+        w64[i] = make_double2(c, s);
+        w32[i] = make_float2((float)c, (float)s);
     }
 }
 
@@ -294,14 +424,21 @@ template <typename T> const T *wmap(akra_plan p);
 template <> const double *wmap<double>(akra_plan p) { return p->d_W64; }
 template <> const float *wmap<float>(akra_plan p) { return p->d_W32; }
 
+template <typename T, int MODE, int LOGN>
+static void launch_rows(const Args<T> &a, int R, cudaStream_t st)
+{
+    constexpr int n = 1 << LOGN, rpb = rows_per_block<T>(n);
+    k_rows<T, MODE, LOGN><<<dim3(n / rpb, R), rpb * (n / 16), rpb * slots(n) * sizeof(cx_t<T>), st>>>(a);
+}
+
 template <typename T, int MODE>
-static akra_status rows(akra_plan p, const void *in, void *out, int R, const void *xreg, double lam,
+static akra_status rows(akra_plan p, const void *in, void *out, bool tr, int R, const void *xreg, double lam,
                         double scale, cudaStream_t st)
 {
     Args<T> a{};
-    a.n = p->nside;
-    a.logn = p->flat_logn;
-    a.w = twiddles<T>(p);
+    a.tr = tr;
+    a.wb = twiddles<T>(p);
+    a.wf = a.wb + p->nside;
     a.in = (const cx_t<T> *)in;
     a.out = (cx_t<T> *)out;
     a.Wt = wt<T>(p);
@@ -309,8 +446,18 @@ static akra_status rows(akra_plan p, const void *in, void *out, int R, const voi
     a.lam = (T)lam;
     a.scale = (T)scale;
     a.skip = p->cur_skip;
-    const size_t smem = (size_t)slots(a.n) * sizeof(cx_t<T>);
-    k_rows<T, MODE><<<dim3(a.n, R), NT, smem, st>>>(a);
+    switch (p->flat_logn) {
+    case 4: launch_rows<T, MODE, 4>(a, R, st); break;
+    case 5: launch_rows<T, MODE, 5>(a, R, st); break;
+    case 6: launch_rows<T, MODE, 6>(a, R, st); break;
+    case 7: launch_rows<T, MODE, 7>(a, R, st); break;
+    case 8: launch_rows<T, MODE, 8>(a, R, st); break;
+    case 9: launch_rows<T, MODE, 9>(a, R, st); break;
+    case 10: launch_rows<T, MODE, 10>(a, R, st); break;
+    case 11: launch_rows<T, MODE, 11>(a, R, st); break;
+    case 12: launch_rows<T, MODE, 12>(a, R, st); break;
+    default: launch_rows<T, MODE, 13>(a, R, st); break;
+    }
     AKRA_CUDA_TRY(cudaGetLastError());
     p->launches++;
     return AKRA_OK;
@@ -326,6 +473,15 @@ static akra_status transpose(akra_plan p, const void *in, void *out, int R, cuda
     return AKRA_OK;
 }
 
+// a pass whose result is wanted transposed; tmp (as large) is used where the store does not transpose
+template <typename T, int MODE>
+static akra_status rows_t(akra_plan p, const void *in, void *out, void *tmp, int R, double scale, cudaStream_t st)
+{
+    if (fused_transpose(p->nside)) return rows<T, MODE>(p, in, out, true, R, nullptr, 0.0, scale, st);
+    AKRA_TRY((rows<T, MODE>(p, in, tmp, false, R, nullptr, 0.0, scale, st)));
+    return transpose<T>(p, tmp, out, R, st);
+}
+
 template <typename T>
 static akra_status buffers(akra_plan p, int R, cx_t<T> **b1, cx_t<T> **b2)
 {
@@ -336,6 +492,36 @@ static akra_status buffers(akra_plan p, int R, cx_t<T> **b1, cx_t<T> **b2)
     return AKRA_OK;
 }
 
+// the shared-memory opt-in of the row kernels that take more than 48 KB (at plan creation, never inside a capture)
+template <typename T, int MODE, int LOGN>
+static cudaError_t prepare_one()
+{
+    constexpr int n = 1 << LOGN, bytes = rows_per_block<T>(n) * slots(n) * (int)sizeof(cx_t<T>);
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(k_rows<T, MODE, LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+template <typename T, int MODE> static cudaError_t prepare_mode()
+{
+    cudaError_t e = prepare_one<T, MODE, 11>();
+    if (e == cudaSuccess) e = prepare_one<T, MODE, 12>();
+    if (e == cudaSuccess) e = prepare_one<T, MODE, 13>();
+    return e;
+}
+template <typename T> static cudaError_t prepare_type()
+{
+    cudaError_t e = prepare_mode<T, 0>();
+    if (e == cudaSuccess) e = prepare_mode<T, 1>();
+    if (e == cudaSuccess) e = prepare_mode<T, 2>();
+    if (e == cudaSuccess) e = prepare_mode<T, 3>();
+    if (e == cudaSuccess) e = prepare_mode<T, 4>();
+    return e;
+}
+static cudaError_t rows_prepare()
+{
+    const cudaError_t e = prepare_type<float>();
+    return e == cudaSuccess ? prepare_type<double>() : e;
+}
+
 }  // namespace flat
 
 template <typename T>
@@ -344,10 +530,9 @@ akra_status flat_op_A(akra_plan p, const void *x, void *map, bool weighted, int 
     cx_t<T> *b1, *b2;
     AKRA_TRY(flat::buffers<T>(p, R, &b1, &b2));
     const double s = 1.0 / (double)p->nside;
-    AKRA_TRY((flat::rows<T, 0>(p, x, b1, R, nullptr, 0.0, 1.0, st)));   // ×D, inverse along k1
-    AKRA_TRY(flat::transpose<T>(p, b1, b2, R, st));
-    AKRA_TRY((flat::rows<T, 3>(p, b2, b2, R, nullptr, 0.0, s, st)));   // inverse along k2, × 1/n
-    AKRA_TRY(flat::transpose<T>(p, b2, b1, R, st));
+    AKRA_TRY((flat::rows_t<T, 0>(p, x, b2, b1, R, 1.0, st)));   // ×D, inverse along k1; [x][k2]
+    // inverse along k2, × 1/n; [y][x].  In place where the store transposes separately
+    AKRA_TRY((flat::rows_t<T, 3>(p, b2, b1, b2, R, s, st)));
     flat::k_split<T><<<1216, 256, 0, st>>>(p->npix, R, b1, weighted ? flat::wmap<T>(p) : nullptr, (T *)map);
     AKRA_CUDA_TRY(cudaGetLastError());
     p->launches++;
@@ -363,9 +548,8 @@ akra_status flat_op_At(akra_plan p, const void *map, void *x, bool weighted, int
     AKRA_CUDA_TRY(cudaGetLastError());
     p->launches++;
     AKRA_TRY(flat::transpose<T>(p, b1, b2, R, st));                            // [x][y]
-    AKRA_TRY((flat::rows<T, 4>(p, b2, b2, R, nullptr, 0.0, 1.0, st)));        // forward along y
-    AKRA_TRY(flat::transpose<T>(p, b2, b1, R, st));                            // [k2][x]
-    return flat::rows<T, 2>(p, b1, x, R, nullptr, 0.0, 1.0 / (double)p->nside, st);   // along x, ×conj D / n
+    AKRA_TRY((flat::rows_t<T, 4>(p, b2, b1, b2, R, 1.0, st)));                 // forward along y; [k2][x]
+    return flat::rows<T, 2>(p, b1, x, false, R, nullptr, 0.0, 1.0 / (double)p->nside, st);   // along x, ×conj D / n
 }
 
 template <typename T>
@@ -373,11 +557,9 @@ akra_status flat_op_H(akra_plan p, const void *x, void *y, int R, cudaStream_t s
 {
     cx_t<T> *b1, *b2;
     AKRA_TRY(flat::buffers<T>(p, R, &b1, &b2));
-    AKRA_TRY((flat::rows<T, 0>(p, x, b1, R, nullptr, 0.0, 1.0, st)));        // ×D, inverse along k1
-    AKRA_TRY(flat::transpose<T>(p, b1, b2, R, st));
-    AKRA_TRY((flat::rows<T, 1>(p, b2, b2, R, nullptr, 0.0, 1.0, st)));       // along k2: F^-1, ×W/n², F
-    AKRA_TRY(flat::transpose<T>(p, b2, b1, R, st));
-    return flat::rows<T, 2>(p, b1, y, R, x, p->lambda_eff, 1.0, st);          // along x, ×conj D, + λ x
+    AKRA_TRY((flat::rows_t<T, 0>(p, x, b2, b1, R, 1.0, st)));        // ×D, inverse along k1; [x][k2]
+    AKRA_TRY((flat::rows_t<T, 1>(p, b2, b1, b2, R, 1.0, st)));       // along k2: F^-1, ×W/n², F; [k2][x]
+    return flat::rows<T, 2>(p, b1, y, false, R, x, p->lambda_eff, 1.0, st);   // along x, ×conj D, + λ x
 }
 
 template akra_status flat_op_A<float>(akra_plan, const void *, void *, bool, int, cudaStream_t);
@@ -455,28 +637,29 @@ extern "C" akra_status akra_flat_plan_create(int n, akra_plan *out)
         akra_plan_destroy(p);
         return AKRA_ENOMEM;
     };
-    if (cudaMalloc(&p->d_ftw64, sizeof(double2) * n) != cudaSuccess ||
-        cudaMalloc(&p->d_ftw32, sizeof(float2) * n) != cudaSuccess ||
+    if (cudaMalloc(&p->d_ftw64, sizeof(double2) * 2 * n) != cudaSuccess ||
+        cudaMalloc(&p->d_ftw32, sizeof(float2) * 2 * n) != cudaSuccess ||
         cudaMalloc(&p->d_W64, sizeof(double) * np) != cudaSuccess ||
         cudaMalloc(&p->d_W32, sizeof(float) * np) != cudaSuccess ||
         cudaMalloc(&p->d_fWt64, sizeof(double) * np) != cudaSuccess ||
         cudaMalloc(&p->d_fWt32, sizeof(float) * np) != cudaSuccess)
         return fail("table allocation failed");
-    p->bytes_tables = (sizeof(double2) + sizeof(float2)) * n + 2 * (sizeof(double) + sizeof(float)) * np;
-    flat::k_twiddles<<<(n + 255) / 256, 256>>>(n, p->d_ftw64, p->d_ftw32);
+    p->bytes_tables = (sizeof(double2) + sizeof(float2)) * 2 * n + 2 * (sizeof(double) + sizeof(float)) * np;
+    // twiddles of the backward passes (R0, 16, 16, ..) from 0, of the forward ones (16, .., R0) from n
+    const int r0 = 1 << (lg & 3);
+    for (int dir = 0; dir < 2; dir++) {
+        int off = dir * n;
+        for (int Ns = dir == 0 ? r0 : 1; Ns < (dir == 0 ? n : n / r0); Ns *= 16) {
+            if (Ns == 1) continue;   // no twiddles
+            flat::k_twiddles<<<(15 * Ns + 255) / 256, 256>>>(Ns, 16, p->d_ftw64 + off, p->d_ftw32 + off);
+            off += 15 * Ns;
+        }
+        if (dir == 1 && r0 > 1 && n / r0 > 1)
+            flat::k_twiddles<<<((r0 - 1) * (n / r0) + 255) / 256, 256>>>(n / r0, r0, p->d_ftw64 + off, p->d_ftw32 + off);
+    }
     cudaError_t e = cudaGetLastError();
-    // row kernels: shared memory for the largest supported row, set once for every plan
-    const int s64 = flat::slots(flat::kMaxN) * (int)sizeof(double2), s32 = flat::slots(flat::kMaxN) * (int)sizeof(float2);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<double, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<double, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<float, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<float, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, s32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, s32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, s32);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(flat::k_rows<float, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s32);
+    // row kernels: shared memory of the largest block, set once for every plan
+    if (e == cudaSuccess) e = flat::rows_prepare();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_a, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_b, cudaEventDisableTiming);

@@ -310,7 +310,7 @@ struct akra_plan_s {
     int *d_all_rings = nullptr;              // [nring] 0..nring-1
     int *d_all_units = nullptr;              // [nunit] 0..nunit-1
 
-    // flat-sky plan: twiddles e^{-2πi t/n}, weights W = M N^-1 transposed and scaled by 1/n^2
+    // flat-sky plan: twiddles of the row passes (backward, then forward), weights W = M N^-1 transposed and scaled by 1/n^2
     int flat_logn = 0;
     double2 *d_ftw64 = nullptr;
     float2 *d_ftw32 = nullptr;
