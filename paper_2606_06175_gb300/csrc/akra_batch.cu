@@ -286,15 +286,19 @@ static akra_status batch_H32(akra_batch b, void *const *x, void *const *y, const
         AKRA_TRY(launch_queue(b, 0, st));
         AKRA_TRY(batch_blk(b, 0, x, skips, st));
     }
-    const size_t smem = (size_t)(f32_slots(b->fft_mmax) + F32_NT) * sizeof(float2);
-    if (smem > b->fft_smem_set) {
+    const int nt = f32_threads(b->fft_mmax, b->nfitems);
+    const size_t smem = (size_t)(f32_slots(b->fft_mmax) + nt) * sizeof(float2);
+    if (nt == F32_NT && smem > b->fft_smem_set) {   // smaller blocks stay below 48 KB
         // the attribute belongs to this translation unit's instance of the kernel
-        AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32_batch<2, F32_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)smem));
         b->fft_smem_set = smem;
     }
     if (b->nfitems > 0) {
-        k_ring_fft32_batch<2><<<b->nfitems, F32_NT, smem, st>>>(b->d_fft, b->d_fitems, b->fft_mmax);
+        if (nt == 64) k_ring_fft32_batch<2, 64><<<b->nfitems, nt, smem, st>>>(b->d_fft, b->d_fitems, b->fft_mmax);
+        else if (nt == 128) k_ring_fft32_batch<2, 128><<<b->nfitems, nt, smem, st>>>(b->d_fft, b->d_fitems, b->fft_mmax);
+        else if (nt == 256) k_ring_fft32_batch<2, 256><<<b->nfitems, nt, smem, st>>>(b->d_fft, b->d_fitems, b->fft_mmax);
+        else k_ring_fft32_batch<2, F32_NT><<<b->nfitems, nt, smem, st>>>(b->d_fft, b->d_fitems, b->fft_mmax);
         AKRA_CUDA_TRY(cudaGetLastError());
         b->launches++;
     }

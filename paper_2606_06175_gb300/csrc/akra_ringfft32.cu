@@ -61,6 +61,15 @@ static int next_pow2(int v)
     return m;
 }
 
+// kernel attributes are shared by every plan: the largest block of each thread count
+template <int MODE>
+static akra_status prepare_item()
+{
+    const int smem = (f32_slots(F32_MMAX) + F32_NT) * (int)sizeof(float2);
+    AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32<MODE, F32_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return AKRA_OK;   // the smaller blocks stay below 48 KB
+}
+
 // plan tables of the FP32 ring FFT (convolution lengths, chirp spectra, pow2 twiddles)
 akra_status ring_fft32_build(akra_plan p)
 {
@@ -106,19 +115,15 @@ akra_status ring_fft32_build(akra_plan p)
     AKRA_CUDA_TRY(cudaMemcpy(p->d_fft32_off, off.data(), sizeof(long long) * (N + 1), cudaMemcpyHostToDevice));
     k_tw2<<<(F32_MMAX + 255) / 256, 256>>>(p->d_fft32_tw2);
     AKRA_CUDA_TRY(cudaGetLastError());
-    // kernel attributes are shared by every plan: clear the largest supported length
     const int smem_b = f32_slots(mmax) * (int)sizeof(float2);
     AKRA_CUDA_TRY(cudaFuncSetAttribute(k_bhat32, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        f32_slots(F32_MMAX) * (int)sizeof(float2)));
     k_bhat32<<<N, F32_NT, smem_b>>>(N, p->d_fft32_M, p->d_fft32_off, p->d_tw64, p->d_fft32_tw2,
                                     p->d_fft32_bhat);
     AKRA_CUDA_TRY(cudaGetLastError());
-    const int smem = (f32_slots(F32_MMAX) + F32_NT) * (int)sizeof(float2);
-    AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    AKRA_CUDA_TRY(cudaFuncSetAttribute(k_ring_fft32_batch<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (f32_slots(F32_MMAX) + F32_NT) * (int)sizeof(float2)));
+    AKRA_TRY(prepare_item<0>());
+    AKRA_TRY(prepare_item<1>());
+    AKRA_TRY(prepare_item<2>());
     return AKRA_OK;
 }
 
@@ -162,13 +167,23 @@ Fft32Args fft32_args(akra_plan p, bool weighted, const int *rings)
     return a;
 }
 
+template <int MODE>
+static void launch_item(const Fft32Args &a, int nt, dim3 grid, size_t smem, cudaStream_t st)
+{
+    if (nt == 64) k_ring_fft32<MODE, 64><<<grid, 64, smem, st>>>(a);
+    else if (nt == 128) k_ring_fft32<MODE, 128><<<grid, 128, smem, st>>>(a);
+    else if (nt == 256) k_ring_fft32<MODE, 256><<<grid, 256, smem, st>>>(a);
+    else k_ring_fft32<MODE, F32_NT><<<grid, F32_NT, smem, st>>>(a);
+}
+
 akra_status ring_fft32(akra_plan p, FftMode mode, void *phi, const void *map_in, void *map_out,
                        bool weighted, int R, const int *rings, int nrings, cudaStream_t st)
 {
     if (nrings <= 0) return AKRA_OK;
     // The plan's own ring lists go out in two launches by convolution length where a block of the larger
     // length reserves so much shared memory that only one fits on an SM (Nside above 1024); below that a
-    // second launch only adds its latency (one H at Nside 32: 28.7 -> 16.0 us, 128: 29.3 -> 20.2, 256: 39 -> 35).
+    // second launch only adds its latency (one H at Nside 32: 28.7 -> 16.0 us, 128: 29.3 -> 20.2,
+    // 256: 39 -> 33).
     const int *list = rings;
     int nsmall = 0;
     const bool split = (size_t)(f32_slots(p->fft32_mmax) + F32_NT) * sizeof(float2) > 100 * 1024;
@@ -188,15 +203,14 @@ akra_status ring_fft32(akra_plan p, FftMode mode, void *phi, const void *map_in,
         if (cnt <= 0) continue;
         a.rings = list + (part == 0 ? 0 : nsmall);
         a.mmax = part == 0 ? p->fft32_msmall : p->fft32_mmax;   // buffer length; scratch follows it
-        const size_t smem = (size_t)(f32_slots(a.mmax) + F32_NT) * sizeof(float2);
+        const int nt = f32_threads(a.mmax, (long long)cnt * R);
+        const size_t smem = (size_t)(f32_slots(a.mmax) + nt) * sizeof(float2);
         dim3 grid(cnt, R);
-#define AKRA_F32_LAUNCH(MD) k_ring_fft32<MD><<<grid, F32_NT, smem, st>>>(a)
         switch (mode) {
-        case FftMode::Synth: AKRA_F32_LAUNCH(0); break;
-        case FftMode::Adjoint: AKRA_F32_LAUNCH(1); break;
-        default: AKRA_F32_LAUNCH(2); break;
+        case FftMode::Synth: launch_item<0>(a, nt, grid, smem, st); break;
+        case FftMode::Adjoint: launch_item<1>(a, nt, grid, smem, st); break;
+        default: launch_item<2>(a, nt, grid, smem, st); break;
         }
-#undef AKRA_F32_LAUNCH
         AKRA_CUDA_TRY(cudaGetLastError());
         p->launches++;
     }

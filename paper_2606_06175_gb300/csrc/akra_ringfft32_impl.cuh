@@ -5,10 +5,30 @@
 
 namespace akra {
 
-constexpr int F32_NT = 512;
+constexpr int F32_NT = 512;               // threads per block at most
 constexpr int F32_MMAX = 8 * kMaxNside;   // largest convolution length (n <= 4 nside - 4)
-constexpr int F32_KPT = 4 * kMaxNside / F32_NT;   // ring pixels per thread at most
+constexpr int F32_KPT = 16;               // ring pixels per thread at most
 static_assert(F32_KPT * F32_NT >= 4 * kMaxNside, "a ring must fit F32_KPT slots per thread");
+// Threads per block for `blocks` rings whose longest convolution is m.  A radix-16 pass has work for m/16 threads
+// and the other loops for up to n, so a ring takes longer on fewer threads, about 1.6 times per halving, but
+// an SM then holds twice the rings (1024 threads at 64 registers): the cheapest product of waves and time per
+// wave.  Measured, us of one H's FFT at (512, 256, 128, 64) threads: 353 rings of Nside 256 37.1, 33.0, 38.8, -;
+// 1023 rings 59.1, 53.1, 46.5, -; 2044 of Nside 128 82.2, 57.8, 55.6, 46.7; 707 of Nside 512 69.7, 83.9; 2047 157.8,
+// 131.1; 177 of Nside 128 20.4, 20.1, 22.7, 28.7.
+inline int f32_threads(int m, long long blocks)
+{
+    int best = F32_NT;
+    double cost = 0, t = 1;
+    for (int nt = F32_NT; nt >= 64 && nt >= m / 16; nt /= 2, t *= 1.6) {
+        const long long slots = 152LL * (1024 / nt);
+        const double c = (double)((blocks + slots - 1) / slots) * t;
+        if (nt == F32_NT || c < cost) {
+            best = nt;
+            cost = c;
+        }
+    }
+    return best;
+}
 
 __device__ __forceinline__ float2 cm(float2 a, float2 b)
 {
@@ -239,7 +259,7 @@ __device__ void bluestein(float2 *x, int n, int M, int logM, const float2 *__res
 
 __device__ __forceinline__ int fdiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-template <int MODE>
+template <int MODE, int NT>
 __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ring, const int r,
                                                 float2 *buf, float2 *red)
 {
@@ -272,8 +292,8 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
 
     if (MODE != (int)FftMode::Adjoint) {
         // fold Φ(m) into n bins: F[k] = e^{iπσk/n} Σ_q (-1)^{σq} Φ(k + nq)
-        if (n >= F32_NT) {
-            // a thread's bins k = tid + u·F32_NT (u < F32_KPT), each summed over q in increasing
+        if (n >= NT) {
+            // a thread's bins k = tid + u·NT (u < F32_KPT), each summed over q in increasing
             // order; the loads of one q are independent, so they are all in flight together
             float2 acc[F32_KPT];
 #pragma unroll
@@ -283,7 +303,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
                 const bool neg = sigma && (q & 1);
 #pragma unroll
                 for (int u = 0; u < F32_KPT; u++) {
-                    const int k = tid + u * F32_NT, m = k + n * q;
+                    const int k = tid + u * NT, m = k + n * q;
                     if (k < n && m >= -L && m <= L) {
                         const float2 v = prow[AKRA_ROW(m)];
                         acc[u] = neg ? csub(acc[u], v) : cadd(acc[u], v);
@@ -292,11 +312,11 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
             }
 #pragma unroll
             for (int u = 0; u < F32_KPT; u++) {
-                const int k = tid + u * F32_NT;
+                const int k = tid + u * NT;
                 if (k < n) buf[pd(k)] = sigma ? cm(acc[u], tw[k]) : acc[u];
             }
         } else {
-            const int G = F32_NT / n, g = tid / n, k = tid - g * n;
+            const int G = NT / n, g = tid / n, k = tid - g * n;
             if (g < G) {
                 const int qlo = -((L + k) / n), qhi = fdiv(L - k, n);
                 float2 acc = make_float2(0.f, 0.f);
@@ -308,7 +328,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
                 red[g * n + k] = acc;
             }
             __syncthreads();
-            for (int kk = tid; kk < n; kk += F32_NT) {
+            for (int kk = tid; kk < n; kk += NT) {
                 float2 acc = make_float2(0.f, 0.f);
                 for (int gg = 0; gg < G; gg++) acc = cadd(acc, red[gg * n + kk]);
                 buf[pd(kk)] = sigma ? cm(acc, tw[kk]) : acc;
@@ -321,7 +341,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
         if (MODE == (int)FftMode::Synth) {
             float *o1 = map_out + ((size_t)r * 2 + 0) * npix + first;
             float *o2 = map_out + ((size_t)r * 2 + 1) * npix + first;
-            for (int k = tid; k < n; k += F32_NT) {
+            for (int k = tid; k < n; k += NT) {
                 const int j = pow2 ? (int)(__brev((unsigned)k) >> (32 - logn)) : k;
                 float2 v = buf[pd(k)];
                 if (weighted) {
@@ -337,7 +357,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
         // ×W: slot k's weight is W[first + k] (stored in this slot order), loads all in flight
 #pragma unroll
         for (int u = 0; u < F32_KPT; u++) {
-            const int k = tid + u * F32_NT;
+            const int k = tid + u * NT;
             if (k < n) {
                 const float wj = W[AKRA_IX(first + k, npix, kDbgFftWeight)];
                 buf[pd(k)].x *= wj;
@@ -348,7 +368,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
     } else {
         const float *u1 = map_in + ((size_t)r * 2 + 0) * npix + first;
         const float *u2 = map_in + ((size_t)r * 2 + 1) * npix + first;
-        for (int k = tid; k < n; k += F32_NT) {
+        for (int k = tid; k < n; k += NT) {
             const int j = pow2 ? (int)(__brev((unsigned)k) >> (32 - logn)) : k;
             float2 v = make_float2(u1[AKRA_PIX(j, kDbgFftMapIn)], u2[AKRA_PIX(j, kDbgFftMapIn)]);
             if (weighted) {
@@ -364,7 +384,7 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
     if (pow2) dit<-1>(buf, n, logn, tw2);
     else bluestein<-1>(buf, n, M, logM, tw, bhat, tw2);
     // unfold: Φ'(m) = e^{-iπσk/n} (-1)^{σq} Ŵ[k],  m = k + nq
-    for (int mm = tid; mm < 2 * L + 1; mm += F32_NT) {
+    for (int mm = tid; mm < 2 * L + 1; mm += NT) {
         const int m = mm - L;
         const int q = fdiv(m, n), k = m - q * n;
         float2 v = buf[pd(k)];
@@ -379,28 +399,28 @@ __device__ __forceinline__ void ring_fft32_item(const Fft32Args &a, const int ri
 }
 
 
-template <int MODE>
-__global__ void __launch_bounds__(F32_NT, 2) k_ring_fft32(Fft32Args a)
+template <int MODE, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_ring_fft32(Fft32Args a)
 {
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *buf = reinterpret_cast<float2 *>(smem_raw);
     const int ring = a.rings ? a.rings[blockIdx.x] : (int)blockIdx.x;
-    ring_fft32_item<MODE>(a, ring, blockIdx.y, buf, buf + f32_slots(a.mmax));
+    ring_fft32_item<MODE, NT>(a, ring, blockIdx.y, buf, buf + f32_slots(a.mmax));
 }
 
 // batched form over several plans: item = {instance, index into its ring list, RHS, 0}
-template <int MODE>
-__global__ void __launch_bounds__(F32_NT)
+template <int MODE, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
 k_ring_fft32_batch(const Fft32Args *__restrict__ insts, const int4 *__restrict__ items, int mmax)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *buf = reinterpret_cast<float2 *>(smem_raw);
     const int4 w = items[blockIdx.x];
-    const Fft32Args a = insts[w.x];
+    const Fft32Args &a = insts[w.x];
     if (a.skip && *a.skip) return;
     const int ring = a.rings ? a.rings[w.y] : w.y;
-    ring_fft32_item<MODE>(a, ring, w.z, buf, buf + f32_slots(mmax));
+    ring_fft32_item<MODE, NT>(a, ring, w.z, buf, buf + f32_slots(mmax));
 }
 
 }  // namespace akra
