@@ -164,12 +164,18 @@ akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const v
 {
     if (nunits <= 0) return AKRA_OK;
     if constexpr (std::is_same<T, float>::value) {
-        if (s.TC > 0) return legendre_synth_tc(p, s.TC, mode, alm, phi, R, units, nunits, st);
-        if (s.BS && blk_pays(p, units, false)) {
+        // Groups of 4 and 8 RHS leave the tensor-core GEMM's columns thin: on one-ring lists the block-jump kernel,
+        // whose own contractions are on the tensor cores, takes them too.  Synthesis, ms, groups -> block jumps:
+        // (1024, 2048) 8 RHS of 4 12.7, of 8 9.17 -> 5.42; (512, 1024) 1.79, 1.32 -> 0.95.  16 RHS of 16 10.3
+        // against 10.8 and 1.55 against 1.89: larger groups stay.
+        const bool jump = s.BS && blk_pays(p, units, false);
+        if (s.TC > 0 && !(jump && s.TC <= 8 && blk_pays(p, units, true)))
+            return legendre_synth_tc(p, s.TC, mode, alm, phi, R, units, nunits, st);
+        if (jump) {
             // the polar ring pairs (the first of the list) keep the difference-form kernels
             const int npolar = blk_tables(p, units).npolar;
             LegShape sp = s;
-            sp.BS = 0;
+            sp.BS = sp.TC = 0;
             AKRA_TRY(legendre_synth<T>(p, sp, mode, alm, phi, R, units, npolar, st));
             return legendre_synth_blk(p, mode, alm, phi, R, units, st);
         }

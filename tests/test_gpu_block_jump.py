@@ -64,3 +64,29 @@ def test_block_jump_propagates_non_finite_values():
         xx[0, 0, O.tri_index(L, 3, 100)] = bad
         assert not bool(torch.isfinite(torch.view_as_real(A.akra_apply_H(p, A.F32, xx))).all())
     assert bool((A.akra_apply_H(p, A.F32, torch.zeros_like(x)) == 0).all())
+
+
+@pytest.mark.parametrize("N,L,R,group", [(64, 128, 1, 4), (64, 128, 9, 8), (100, 257, 3, 8), (64, 127, 3, 8), (64, 128, 9, 16)])
+def test_tensor_core_groups_on_one_ring_footprints(N, L, R, group):
+    """Groups of 4 and 8 take the block-jump kernel from lmax 128 on, larger ones and smaller lmax do not; a fixed
+    shape keeps the group's own kernel."""
+    rng = np.random.default_rng(L + R)
+    z = np.cos(O.pixel_angles(N)[0])
+    ninv = np.where(SKIES["south"](z), 1.0 + rng.random(12 * N * N), 0.0)
+    w = O.Weights(N, ninv, 1e-3)
+    p = A.akra_plan_create(N, L)
+    A.akra_plan_set_weights(p, torch.from_numpy(ninv).to(DEV), 1e-3)
+    pairs = [(S.random_alm(L, rng), S.random_alm(L, rng)) for _ in range(R)]
+    x = torch.from_numpy(np.stack([np.stack(q) for q in pairs])).to(DEV, torch.complex64)
+    plain = A.akra_apply_H(p, A.F32, x)
+    A.akra_plan_set_tc_synthesis(p, R, group)
+    assert A.akra_plan_get_tc_synthesis(p, R) == group
+    y = A.akra_apply_H(p, A.F32, x)
+    assert torch.equal(y, plain) == (group <= 8 and L >= 128)
+    A.akra_plan_set_shape(p, A.F32, R, 1, 1, 1)
+    A.akra_plan_set_tc_synthesis(p, R, group)
+    fixed = A.akra_apply_H(p, A.F32, x)
+    for r in range(R):
+        ref = np.stack(O.apply_H(N, L, w, *pairs[r]))
+        assert rel(y[r].cpu().numpy(), ref) < tol32(L), ("H", r)
+        assert rel(fixed[r].cpu().numpy(), ref) < tol32(L), ("fixed shape", r)
