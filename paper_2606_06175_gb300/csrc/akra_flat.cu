@@ -12,7 +12,8 @@
 // reads rows again, and for H the second and third passes (inverse along y, ×W, forward along y) are one
 // kernel per row of the transposed field, as the ring FFT fuses W between its two DFTs.
 //
-// Row FFTs are radix-16 Stockham passes (plus one pass of radix 2, 4 or 8 where log2 n is no multiple of 4),
+// Row FFTs are radix-16 Stockham passes (plus one pass of radix 2, 4 or 8 where log2 n is no multiple of 4; radix 4
+// for FP64 rows up to 256),
 // 16 elements of a row in each thread's registers: a row of 2048 crosses shared memory twice instead of the
 // six times of radix-4 passes, consecutive threads load consecutive twiddles, and the first pass reads and the
 // last writes global memory directly.  n is a template argument, which leaves one address and immediate
@@ -97,17 +98,23 @@ template <int S, typename T, int R> __device__ __forceinline__ void dft(cx_t<T> 
     }
 }
 
-// A row of N = 2^LOGN in N/16 threads: radix-16 passes and one of R0 = 2^(LOGN mod 4) where that is not 1.  Everything
-// but the thread's index is a compile-time constant, so that the accesses of a pass are one address and
-// immediate offsets.
+// log2 of the elements E of a row in a thread: 16 elements and radix-16 passes, but 4 for the FP64 rows up to 256,
+// whose few warps are bound by each warp's own FP64 instructions (H at n = 64: 70 us with 16, 27 with 4;
+// 39 with radix-4 passes through shared memory).
+template <typename T> __host__ __device__ constexpr int log_elems(int logn) { return sizeof(T) == 8 && logn <= 8 ? 2 : 4; }
+
+// A row of N = 2^LOGN in N/E threads: radix-E passes and one of R0 = 2^(LOGN mod log2 E) where that is not 1.
+// Everything but the thread's index is a compile-time constant, so that the accesses of a pass are one
+// address and immediate offsets.
 template <typename T, int LOGN>
 struct Row {
     using C = cx_t<T>;
-    static constexpr int N = 1 << LOGN, TN = N / 16, R0 = 1 << (LOGN & 3);
-    static constexpr int R1 = R0 > 1 ? R0 : 16;   // first pass of the backward transform, last of the forward one
+    static constexpr int LE = log_elems<T>(LOGN), E = 1 << LE;
+    static constexpr int N = 1 << LOGN, TN = N / E, R0 = 1 << (LOGN % LE);
+    static constexpr int R1 = R0 > 1 ? R0 : E;   // first pass of the backward transform, last of the forward one
 
     // offset from t of the place of v[i] as the first pass of radix R reads it and the last one leaves it
-    template <int R> static __host__ __device__ constexpr int place(int i) { return (i / R) * TN + (i % R) * (16 / R) * TN; }
+    template <int R> static __host__ __device__ constexpr int place(int i) { return (i / R) * TN + (i % R) * (E / R) * TN; }
 
     // slot of element i + off
     static __device__ __forceinline__ int at(int i, int off)
@@ -115,13 +122,13 @@ struct Row {
         return off % 16 == 0 ? pd(i) + off + off / 16 : pd(i + off);
     }
 
-    // Stockham pass of radix R after passes of product Ns: butterflies j = t + u TN (u < 16/R), inputs
+    // Stockham pass of radix R after passes of product Ns: butterflies j = t + u TN (u < E/R), inputs
     // x[j + q N/R] in v[u R + q], twiddled by e^{S 2πi qk/(Ns R)}, k = j mod Ns (table w[(q - 1) Ns + k],
     // sign -), outputs x[(j - k) R + k + r Ns]
-    template <int S, int R, int Ns> static __device__ __forceinline__ void pass(C (&v)[16], int t, const C *__restrict__ w)
+    template <int S, int R, int Ns> static __device__ __forceinline__ void pass(C (&v)[E], int t, const C *__restrict__ w)
     {
 #pragma unroll
-        for (int u = 0; u < 16 / R; u++) {
+        for (int u = 0; u < E / R; u++) {
             if (Ns > 1) {
                 const C *wk = w + ((t + u * TN) & (Ns - 1));
 #pragma unroll
@@ -135,10 +142,10 @@ struct Row {
         }
     }
     // its outputs to the row's buffer; (k + r Ns) / 16 = r Ns / 16 for every pass
-    template <int R, int Ns> static __device__ __forceinline__ void put(C *buf, const C (&v)[16], int t)
+    template <int R, int Ns> static __device__ __forceinline__ void put(C *buf, const C (&v)[E], int t)
     {
 #pragma unroll
-        for (int u = 0; u < 16 / R; u++) {
+        for (int u = 0; u < E / R; u++) {
             const int k = (t + u * TN) & (Ns - 1);
             const int o = Ns == 1 ? at(t * R, u * TN * R) : pd((t + u * TN - k) * R + k);
 #pragma unroll
@@ -146,44 +153,44 @@ struct Row {
         }
     }
     // inputs of a pass of radix R
-    template <int R> static __device__ __forceinline__ void get(const C *buf, C (&v)[16], int t)
+    template <int R> static __device__ __forceinline__ void get(const C *buf, C (&v)[E], int t)
     {
 #pragma unroll
-        for (int i = 0; i < 16; i++) v[i] = buf[at(t, place<R>(i))];
+        for (int i = 0; i < E; i++) v[i] = buf[at(t, place<R>(i))];
     }
 
-    // radix-16 passes from Ns to the product M; then the buffer holds the inputs of a pass of radix R0, or v the row
-    template <int S, int Ns, int M> static __device__ __forceinline__ void passes16(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    // radix-E passes from Ns to the product M; then the buffer holds the inputs of a pass of radix R0, or v the row
+    template <int S, int Ns, int M> static __device__ __forceinline__ void passes(C (&v)[E], C *buf, int t, const C *__restrict__ w)
     {
         if constexpr (Ns < M) {
-            pass<S, 16, Ns>(v, t, w);
-            if constexpr (Ns * 16 < N) {
+            pass<S, E, Ns>(v, t, w);
+            if constexpr (Ns * E < N) {
                 __syncthreads();   // the buffer's last readers
-                put<16, Ns>(buf, v, t);
+                put<E, Ns>(buf, v, t);
                 __syncthreads();
-                if constexpr (Ns * 16 < M) get<16>(buf, v, t);
+                if constexpr (Ns * E < M) get<E>(buf, v, t);
             }
-            passes16<S, Ns * 16, M>(v, buf, t, w + (Ns > 1 ? 15 * Ns : 0));
+            passes<S, Ns * E, M>(v, buf, t, w + (Ns > 1 ? (E - 1) * Ns : 0));
         } else if constexpr (M < N) {
             get<R0>(buf, v, t);
             pass<S, R0, M>(v, t, w);
         }
     }
-    // Backward: R0, 16, 16, ..; forward: 16, 16, .., R0.  The backward transform ends and the forward one starts
-    // with the same radix-16 places, so ×W between them needs no exchange.
-    static __device__ __forceinline__ void backward(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    // Backward: R0, E, E, ..; forward: E, E, .., R0.  The backward transform ends and the forward one starts
+    // with the same radix-E places, so ×W between them needs no exchange.
+    static __device__ __forceinline__ void backward(C (&v)[E], C *buf, int t, const C *__restrict__ w)
     {
         if constexpr (R0 > 1) {
             pass<+1, R0, 1>(v, t, w);
             put<R0, 1>(buf, v, t);
             __syncthreads();
-            get<16>(buf, v, t);
+            get<E>(buf, v, t);
         }
-        passes16<+1, R0, N>(v, buf, t, w);
+        passes<+1, R0, N>(v, buf, t, w);
     }
-    static __device__ __forceinline__ void forward(C (&v)[16], C *buf, int t, const C *__restrict__ w)
+    static __device__ __forceinline__ void forward(C (&v)[E], C *buf, int t, const C *__restrict__ w)
     {
-        passes16<-1, 1, N / R0>(v, buf, t, w);
+        passes<-1, 1, N / R0>(v, buf, t, w);
     }
 };
 
@@ -215,35 +222,41 @@ __host__ __device__ constexpr bool fused_transpose(int n) { return n <= 4096; }
 
 // Rows of a block.  A transposed store joins 32 bytes, a sector, from 4 FP32 rows: at n = 2048 H takes 95 us against
 // 100 with two, at 4096 (1024 threads) 361 against 425.  FP64 blocks are of 256 threads where that holds a row: at
-// 4096 one row takes 6.03 ms against 6.43 with two, the FP64 pipe being the bound.  Short rows fill 128 threads.
-template <typename T> __host__ __device__ constexpr int rows_per_block(int n)
+// 4096 one row takes 6.03 ms against 6.43 with two, the FP64 pipe being the bound.  Short rows fill a warp: the few
+// blocks of a small grid would otherwise leave most SMs idle.
+template <typename T> __host__ __device__ constexpr int rows_per_block(int logn)
 {
+    const int n = 1 << logn, per_row = n >> log_elems<T>(logn);
     const int sector = 32 / (int)sizeof(cx_t<T>), threads = sizeof(T) == 8 ? 256 : fused_transpose(n) ? 1024 : 512;
-    const int most = threads * 16 / n < 1 ? 1 : threads * 16 / n, least = 128 * 16 / n < n ? 128 * 16 / n : n;
+    const int most = threads < per_row ? 1 : threads / per_row;
+    const int least = per_row >= 32 ? 1 : 32 / per_row < n ? 32 / per_row : n;
     const int rows = sector < most ? sector : most;
     return least > rows ? least : rows;
 }
 
-template <typename T> __host__ __device__ constexpr int row_threads(int n) { return rows_per_block<T>(n) * (n / 16); }
-
-// Registers: 64 a thread in FP32 (1024 threads per SM; 768 take 101 us for H at 2048, where 1024 take 95), 128 in FP64.
-template <typename T> constexpr int row_blocks(int n)
+template <typename T> __host__ __device__ constexpr int row_threads(int logn)
 {
-    return (sizeof(T) == 4 ? 1024 : 512) / (row_threads<T>(n) < 128 ? 128 : row_threads<T>(n));
+    return rows_per_block<T>(logn) * ((1 << logn) >> log_elems<T>(logn));
 }
 
-// rows_per_block rows of one RHS per block, n/16 threads a row.  MODE
+// Registers: 64 a thread in FP32 (1024 threads per SM; 768 take 101 us for H at 2048, where 1024 take 95), 128 in FP64.
+template <typename T> constexpr int row_blocks(int logn)
+{
+    return (sizeof(T) == 4 ? 1024 : 512) / (row_threads<T>(logn) < 128 ? 128 : row_threads<T>(logn));
+}
+
+// rows_per_block rows of one RHS per block, n/E threads a row.  MODE
 //   0: ×D(k1 = column, k2 = row), inverse FFT along the row
 //   1: inverse FFT, ×Wt[row][y], forward FFT (the transposed middle of H)
 //   2: forward FFT, then ×conj(D(k1 = column, k2 = row)) × scale + λ x
 //   3: inverse FFT, × scale
 //   4: forward FFT
 template <typename T, int MODE, int LOGN>
-__global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << LOGN)) k_rows(Args<T> a)
+__global__ void __launch_bounds__(row_threads<T>(LOGN), row_blocks<T>(LOGN)) k_rows(Args<T> a)
 {
     using C = cx_t<T>;
     using F = Row<T, LOGN>;
-    constexpr int n = F::N, tn = F::TN, rpb = rows_per_block<T>(n);
+    constexpr int n = F::N, tn = F::TN, E = F::E, rpb = rows_per_block<T>(LOGN);
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lt = threadIdx.x / tn, t = threadIdx.x % tn;
@@ -251,14 +264,14 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << 
     C *buf = reinterpret_cast<C *>(smem_raw) + lt * slots(n);
     const size_t base = ((size_t)blockIdx.y * n + row) * n + t;
     constexpr bool fwd_only = MODE == 2 || MODE == 4;
-    constexpr int RI = fwd_only ? 16 : F::R1;                          // first pass
-    constexpr int RO = MODE == 0 || MODE == 3 ? 16 : F::R1;            // last pass
+    constexpr int RI = fwd_only ? E : F::R1;                          // first pass
+    constexpr int RO = MODE == 0 || MODE == 3 ? E : F::R1;            // last pass
     const T ft = (T)t, fr = (T)(row < n / 2 ? row : row - n);          // frequencies; n/2 is a multiple of tn
     auto fcol = [&](int off) { return ft + (T)(off < n / 2 ? off : off - n); };
-    C v[16];
+    C v[E];
     const C *in = a.in + base;
 #pragma unroll
-    for (int i = 0; i < 16; i++) {
+    for (int i = 0; i < E; i++) {
         const int off = F::template place<RI>(i);
         v[i] = in[off];
         if (MODE == 0) v[i] = cmul(ks<T>(fcol(off), fr), v[i]);
@@ -267,8 +280,8 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << 
     if (MODE == 1) {
         const T *wt = a.Wt + (size_t)row * n + t;
 #pragma unroll
-        for (int i = 0; i < 16; i++) {
-            const T wy = wt[F::template place<16>(i)];
+        for (int i = 0; i < E; i++) {
+            const T wy = wt[F::template place<E>(i)];
             v[i].x *= wy;
             v[i].y *= wy;
         }
@@ -276,14 +289,14 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << 
     if (fwd_only || MODE == 1) F::forward(v, buf, t, a.wf);
     if (MODE == 3) {
 #pragma unroll
-        for (int i = 0; i < 16; i++) {
+        for (int i = 0; i < E; i++) {
             v[i].x *= a.scale;
             v[i].y *= a.scale;
         }
     }
     if (MODE == 2) {
 #pragma unroll
-        for (int i = 0; i < 16; i++) {
+        for (int i = 0; i < E; i++) {
             const int off = F::template place<RO>(i);
             const C d = ks<T>(fcol(off), fr);
             v[i] = cmul(C{d.x, -d.y}, v[i]);
@@ -299,11 +312,11 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << 
     if (MODE == 2 || !a.tr) {
         C *out = a.out + base;
 #pragma unroll
-        for (int i = 0; i < 16; i++) out[F::template place<RO>(i)] = v[i];
+        for (int i = 0; i < E; i++) out[F::template place<RO>(i)] = v[i];
     } else if constexpr (rpb * sizeof(C) >= 16) {
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 16; i++) buf[F::at(t, F::template place<RO>(i))] = v[i];
+        for (int i = 0; i < E; i++) buf[F::at(t, F::template place<RO>(i))] = v[i];
         __syncthreads();
         constexpr int RC = 16 / sizeof(C);   // rows in a 16-byte store
         struct alignas(16) Chunk { C c[RC]; };
@@ -312,7 +325,7 @@ __global__ void __launch_bounds__(row_threads<T>(1 << LOGN), row_blocks<T>(1 << 
         const C *src = reinterpret_cast<const C *>(smem_raw) + r * slots(n);
         C *dst = a.out + ((size_t)blockIdx.y * n + k) * n + blockIdx.x * rpb + r;
 #pragma unroll
-        for (int i = 0; i < 16 / RC; i++) {
+        for (int i = 0; i < E / RC; i++) {
             Chunk o;
 #pragma unroll
             for (int q = 0; q < RC; q++) o.c[q] = src[q * slots(n) + F::at(k, i * tn * RC)];
@@ -402,15 +415,32 @@ __global__ void k_weights(int n, const double *ninv, double *W64, float *W32, do
 }
 
 // twiddles of one pass: w[(q - 1) Ns + k] = e^{-2πi qk/(Ns R)}, 1 <= q < R, k < Ns
-__global__ void k_twiddles(int Ns, int R, double2 *w64, float2 *w32)
+template <typename T>
+__global__ void k_twiddles(int Ns, int R, cx_t<T> *w)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < (R - 1) * Ns) {
         const int q = 1 + i / Ns, k = i % Ns;
         double s, c;
         sincospi(-2.0 * (double)(q * k) / (double)(Ns * R), &s, &c);
-        w64[i] = make_double2(c, s);
-        w32[i] = make_float2((float)c, (float)s);
+        w[i] = cx_t<T>{(T)c, (T)s};
+    }
+}
+
+// the passes' twiddles in order: of the backward transform (R0, E, E, ..) from 0, of the forward one (E, .., R0) from n
+template <typename T>
+static void build_twiddles(int logn, cx_t<T> *w)
+{
+    const int n = 1 << logn, le = log_elems<T>(logn), E = 1 << le, r0 = 1 << (logn % le);
+    for (int dir = 0; dir < 2; dir++) {
+        cx_t<T> *at = w + dir * n;
+        auto pass = [&](int Ns, int R) {
+            if (Ns == 1 || R == 1) return;   // no twiddles
+            k_twiddles<T><<<((R - 1) * Ns + 255) / 256, 256>>>(Ns, R, at);
+            at += (R - 1) * Ns;
+        };
+        for (int Ns = dir == 0 ? r0 : 1; Ns < (dir == 0 ? n : n / r0); Ns *= E) pass(Ns, E);
+        if (dir == 1) pass(n / r0, r0);
     }
 }
 
@@ -427,8 +457,8 @@ template <> const float *wmap<float>(akra_plan p) { return p->d_W32; }
 template <typename T, int MODE, int LOGN>
 static void launch_rows(const Args<T> &a, int R, cudaStream_t st)
 {
-    constexpr int n = 1 << LOGN, rpb = rows_per_block<T>(n);
-    k_rows<T, MODE, LOGN><<<dim3(n / rpb, R), rpb * (n / 16), rpb * slots(n) * sizeof(cx_t<T>), st>>>(a);
+    constexpr int n = 1 << LOGN, rpb = rows_per_block<T>(LOGN);
+    k_rows<T, MODE, LOGN><<<dim3(n / rpb, R), row_threads<T>(LOGN), rpb * slots(n) * sizeof(cx_t<T>), st>>>(a);
 }
 
 template <typename T, int MODE>
@@ -496,7 +526,7 @@ static akra_status buffers(akra_plan p, int R, cx_t<T> **b1, cx_t<T> **b2)
 template <typename T, int MODE, int LOGN>
 static cudaError_t prepare_one()
 {
-    constexpr int n = 1 << LOGN, bytes = rows_per_block<T>(n) * slots(n) * (int)sizeof(cx_t<T>);
+    constexpr int n = 1 << LOGN, bytes = rows_per_block<T>(LOGN) * slots(n) * (int)sizeof(cx_t<T>);
     if (bytes <= 48 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(k_rows<T, MODE, LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
@@ -645,18 +675,8 @@ extern "C" akra_status akra_flat_plan_create(int n, akra_plan *out)
         cudaMalloc(&p->d_fWt32, sizeof(float) * np) != cudaSuccess)
         return fail("table allocation failed");
     p->bytes_tables = (sizeof(double2) + sizeof(float2)) * 2 * n + 2 * (sizeof(double) + sizeof(float)) * np;
-    // twiddles of the backward passes (R0, 16, 16, ..) from 0, of the forward ones (16, .., R0) from n
-    const int r0 = 1 << (lg & 3);
-    for (int dir = 0; dir < 2; dir++) {
-        int off = dir * n;
-        for (int Ns = dir == 0 ? r0 : 1; Ns < (dir == 0 ? n : n / r0); Ns *= 16) {
-            if (Ns == 1) continue;   // no twiddles
-            flat::k_twiddles<<<(15 * Ns + 255) / 256, 256>>>(Ns, 16, p->d_ftw64 + off, p->d_ftw32 + off);
-            off += 15 * Ns;
-        }
-        if (dir == 1 && r0 > 1 && n / r0 > 1)
-            flat::k_twiddles<<<((r0 - 1) * (n / r0) + 255) / 256, 256>>>(n / r0, r0, p->d_ftw64 + off, p->d_ftw32 + off);
-    }
+    flat::build_twiddles<double>(lg, p->d_ftw64);
+    flat::build_twiddles<float>(lg, p->d_ftw32);
     cudaError_t e = cudaGetLastError();
     // row kernels: shared memory of the largest block, set once for every plan
     if (e == cudaSuccess) e = flat::rows_prepare();
