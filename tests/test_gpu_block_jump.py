@@ -90,3 +90,21 @@ def test_tensor_core_groups_on_one_ring_footprints(N, L, R, group):
         ref = np.stack(O.apply_H(N, L, w, *pairs[r]))
         assert rel(y[r].cpu().numpy(), ref) < tol32(L), ("H", r)
         assert rel(fixed[r].cpu().numpy(), ref) < tol32(L), ("fixed shape", r)
+
+
+def test_badly_filled_chunks_keep_the_direct_adjoint_for_several_rhs():
+    """557 rings in three chunks of 256: from 3 RHS on the direct adjoint takes A^T, one RHS the block jumps."""
+    N, L, R = 380, 130, 3
+    z = np.cos(O.pixel_angles(N)[0])
+    ninv = np.where(SKIES["south"](z), 1.0, 0.0)
+    w = O.Weights(N, ninv, 1e-3)
+    p = A.akra_plan_create(N, L)
+    A.akra_plan_set_weights(p, torch.from_numpy(ninv).to(DEV), 1e-3)
+    u = np.random.default_rng(8).normal(size=(R, 2, 12 * N * N)).astype(np.float32)
+    ud = torch.from_numpy(u).to(DEV)
+    b = A.akra_apply_At(p, A.F32, ud, weighted=True).cpu().numpy()
+    one = A.akra_apply_At(p, A.F32, ud[:1], weighted=True).cpu().numpy()
+    ref = np.stack(O.rhs_b(N, L, w, *u[0].astype(np.float64)))
+    assert rel(b[0], ref) < tol32(L) and rel(one[0], ref) < tol32(L)
+    for r in range(1, R):
+        assert rel(b[r], np.stack(O.rhs_b(N, L, w, *u[r].astype(np.float64)))) < tol32(L)
