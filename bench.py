@@ -548,12 +548,16 @@ def main():
     peak = fp32_peak_tflops(sm_count, sm_max)
     work = legendre_flops(desc)
     dom = "legendre_adjoint" if st32["legendre_adjoint"] >= st32["legendre_synth"] else "legendre_synth"
-    kname = {"legendre_adjoint": "k_leg_adjoint<float>", "legendre_synth": "k_leg_synth<float>"}[dom]
+    # where nearly every ring pair needs one ring the block-jump kernels run (and few polar pairs' direct ones)
+    jump = work["steps_one_ring"] >= 0.9 * work["steps"]
+    kname = {"legendre_adjoint": "k_leg_adjoint", "legendre_synth": "k_leg_synth"}[dom] + ("_blk" if jump else "<float>")
     shape = A.akra_plan_get_shape(plan, A.F32, 1)
     rga = A.akra_plan_get_adjoint_shape(plan, A.F32, 1)["RGA"]
     kfull = "%s<float,%d,%d,128>" % ("k_leg_adjoint" if dom == "legendre_adjoint" else "k_leg_synth",
                                      shape["PA"] if dom == "legendre_adjoint" else shape["P"],
                                      rga if dom == "legendre_adjoint" else shape["RG"])
+    if jump:
+        kfull = kname
     achieved = work["model_flops"] / (st32[dom] * 1e-3) / 1e12
     traffic, traffic_note = captured_traffic(kfull)
     f32_meas = A.akra_fma_rate(A.F32)
@@ -571,7 +575,8 @@ def main():
         "flops_per_launch": work["model_flops"], "lm_pair_steps_per_launch": work["steps"],
         "lm_pair_steps_full_triangle": work["steps_full_triangle"],
         "achieved_full_triangle": work["model_flops_full_triangle"] / (st32[dom] * 1e-3) / 1e12,
-        "executed": {"flops_per_launch": work["executed_flops"],
+        # the block-jump kernels execute about 2 FP32 FMA and 16 tensor-core ones per step, uncounted here
+        "executed": None if jump else {"flops_per_launch": work["executed_flops"],
                      "basis": "FMA per step as executed: monic recurrence 2 x 2 FMA; contraction of both "
                               "rings' E and B parts 8 FMA per RHS, 4 for pairs that need one ring (%d of %d "
                               "steps here)" % (work["steps_one_ring"], work["steps"]),
@@ -592,8 +597,8 @@ def main():
                               "executed_achieved": exec64 / (st64[k] * 1e-3) / 1e12,
                               "executed_frac_of_nominal_fp64": exec64 / (st64[k] * 1e-3) / 1e12 / 1.25}
                           for k in ("legendre_synth", "legendre_adjoint")},
-        # counted steps / lane-steps the warps execute at the chosen shapes (start-point spread
-        # within a warp and 64-step tile granularity)
+        # counted steps / lane-steps the direct kernels' warps execute at the chosen shapes (start-point
+        # spread within a warp and 64-step tile granularity)
         "lane_efficiency": {
             "legendre_synth": A.akra_legendre_lane_steps(plan, A.F32, False, shape["P"])["efficiency"],
             "legendre_adjoint": A.akra_legendre_lane_steps(plan, A.F32, True, shape["PA"])["efficiency"]},
@@ -665,10 +670,10 @@ def main():
             e1.record()
             torch.cuda.synchronize()
             h_ms[nm] = e0.elapsed_time(e1) / 10
-        # HBM traffic of one H: 5 passes over the complex field (row FFT in/out, 2 transposes,
-        # fused middle pass, last pass reading x for the λ_eff term) + the weights
+        # HBM traffic of one H: 3 passes over the complex field (the last one also reads x for the λ_eff
+        # term) + the weights, and 2 transposes above n = 4096
         cb = {"fp32": 8, "fp64": 16}
-        trf = {k: (11 * cb[k] + cb[k] // 2) * nf * nf for k in cb}
+        trf = {k: ((7 if nf <= 4096 else 11) * cb[k] + cb[k] // 2) * nf * nf for k in cb}
         hbm = {k: trf[k] / (h_ms[k] * 1e-3) / 1e9 for k in cb}
         flat = dict(solve_summary(inf_f, t_f), n=nf, pixels=nf * nf, h_apply_ms=h_ms, h_traffic_bytes=trf,
                     h_achieved_gbs=hbm, h_frac_of_hbm={k: hbm[k] / HBM_GBS for k in hbm})
