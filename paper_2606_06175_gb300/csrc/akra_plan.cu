@@ -476,12 +476,16 @@ LegShape leg_shape(akra_plan p, akra_prec prec, int R)
         s.RGA = 1;
     }
     s.BS = s.BA = 1;   // the block-jump kernels where they pay (blk_pays)
-    // From 3 RHS on the direct adjoint shares its recurrence between two, and a footprint that fills its chunks
-    // badly stays with it.  A^T, direct -> block jumps, us, 5 RHS: 548 rings in 3 chunks (71 %; Nside 400) lmax 500
-    // 454 -> 493, lmax 800 839 -> 883; 822 in 4 (80 %; 600) lmax 700 1291 -> 1217, lmax 1200 2704 -> 2340; 351 in 2
-    // (69 %; 256) 183 -> 168, few enough for its latency to count.
+    // From 3 RHS on a footprint that fills its chunks badly stays with the direct adjoint, at 5 pairs and one RHS
+    // per block.  A^T, direct -> block jumps, us, 5 RHS: 548 rings in 3 chunks (71 %; Nside 400) lmax 500
+    // 454 -> 493, lmax 800 839 -> 883 (880 at 2 pairs and 2 RHS); 822 in 4 (80 %; 600) lmax 700 1291 -> 1217, lmax
+    // 1200 2704 -> 2340; 351 in 2 (69 %; 256) 183 -> 168, few enough for its latency to count.
     const BlkTables &t = p->blk_act;
-    if (R >= 3 && t.nchunks >= 3 && t.nrows < 0.77 * 256 * t.nchunks) s.BA = 0;
+    if (R >= 3 && p->mostly_one_ring && t.nchunks >= 3 && t.nrows < 0.77 * 256 * t.nchunks) {
+        s.BA = 0;
+        s.PA = 5;
+        s.RGA = 1;
+    }
     return s;
 }
 
