@@ -53,7 +53,8 @@ struct DebugRecord {
 enum DebugSite {
     kDbgUnits = 1, kDbgUnitInfo, kDbgStart, kDbgSeeds, kDbgCoef, kDbgAlm, kDbgKsFactor,
     kDbgPhiWrite, kDbgPhiRead, kDbgPartialWrite, kDbgPartialRead, kDbgAlmOut, kDbgRingActive,
-    kDbgFftPhi, kDbgFftMapIn, kDbgFftMapOut, kDbgFftWeight, kDbgFftRing, kDbgBpre
+    kDbgFftPhi, kDbgFftMapIn, kDbgFftMapOut, kDbgFftWeight, kDbgFftRing, kDbgBpre,
+    kDbgBarrier   // not an index: an mbarrier phase open at the end of its block
 };
 #ifdef AKRA_DEBUG
 static __device__ DebugRecord g_akra_dbg;   // one per translation unit

@@ -76,11 +76,42 @@ __device__ __forceinline__ uint32_t blk_open(uint32_t *s_tmem, BlkBars *bars)
     return *s_tmem;
 }
 
-__device__ __forceinline__ void blk_close(uint32_t tmem)
+// the bounds-checked build also records a barrier whose last phase is still open when the block ends
+template <bool ADJ>
+__device__ __forceinline__ void blk_check_bars(BlkBars *bars, int T)
+{
+#ifdef AKRA_DEBUG
+    if (threadIdx.x != 0) return;
+    auto check = [](uint64_t *bar, int uses) {
+        if (uses > 0 && !tc::mbar_test(bar, (uses - 1) & 1)) dbg_index(-1, 1, kDbgBarrier);
+    };
+    for (int h = 0; h < 2; h++) {
+        const int nb = (T + 1 - h) / 2;   // uses of a barrier that alternates with the tiles
+        check(&bars->ready[h], nb);
+        check(&bars->bfree[h], nb);
+        for (int u = 0; u < 2; u++) {
+            check(&bars->full[h][u], T);
+            check(&bars->empty[h][u], T);
+        }
+        if (!ADJ) continue;
+        check(&bars->yready[h], T);
+        check(&bars->yfree[h], T);
+        check(&bars->full2[h], nb);
+        check(&bars->empty2[h], nb);
+    }
+#else
+    (void)bars;
+    (void)T;
+#endif
+}
+
+template <bool ADJ>
+__device__ __forceinline__ void blk_close(uint32_t tmem, BlkBars *bars, int T)
 {
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    blk_check_bars<ADJ>(bars, T);
     if (threadIdx.x < 32) tc::tmem_dealloc(tmem, 256);
 }
 
@@ -94,7 +125,7 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_synth_blk(LegArgs<float>
     const int m = blockIdx.x / a.blk_chunks;
     uint32_t tiles = 0;
     blk_synth_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tiles, tmem);
-    blk_close(tmem);
+    blk_close<false>(tmem, &bars, (int)tiles);
 }
 
 __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_adjoint_blk(LegArgs<float> a)
@@ -107,7 +138,7 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_adjoint_blk(LegArgs<floa
     const int m = blockIdx.x / a.blk_chunks;
     uint32_t tiles = 0;
     blk_adjoint_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tiles, tmem);
-    blk_close(tmem);
+    blk_close<true>(tmem, &bars, (int)tiles);
 }
 
 }  // namespace

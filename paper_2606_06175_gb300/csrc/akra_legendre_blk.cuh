@@ -314,6 +314,19 @@ __device__ __forceinline__ bool blk_wait(const LegArgs<float> &a, uint64_t *bar,
 {
     return tc::mbar_wait(bar, use & 1, kBlkWaitLimit, a.err);
 }
+// The item's last arrivals at bfree (and, in the adjoint, at yfree) come from the tensor core's completions and
+// have no other waiter: waited for here by the thread that issued them, so that none is in flight when the block
+// gives its shared memory back (to a block that initialises barriers at the same addresses).
+template <bool ADJ>
+__device__ __forceinline__ bool blk_drain(const LegArgs<float> &a, BlkBars *bars, uint32_t end, int T, int h)
+{
+    bool ok = true;
+    if (T > 0) ok &= blk_wait(a, &bars->bfree[(end - 1) & 1], (end - 1) >> 1);
+    if (T > 1) ok &= blk_wait(a, &bars->bfree[end & 1], (end - 2) >> 1);
+    if (ADJ && T > 0) ok &= blk_wait(a, &bars->yfree[h], end - 1);
+    return ok;
+}
+
 __device__ __forceinline__ void blk_warp_arrive(uint64_t *bar)
 {
     __syncwarp();
@@ -452,6 +465,7 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
                 }
                 tc::commit(&bars->bfree[gt & 1]);
             }
+            ok &= blk_drain<false>(a, bars, tiles + T, T, h);
         }
     } else {
         float4 *s_al = reinterpret_cast<float4 *>(smem + S::OFF_PA);
@@ -792,6 +806,7 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
                     tc::commit(&bars->full2[pt & 1]);
                 }
             }
+            ok &= blk_drain<true>(a, bars, tiles + T, T, h);
         }
     } else {
 #pragma unroll

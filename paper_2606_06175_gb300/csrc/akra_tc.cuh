@@ -107,6 +107,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, int l
     return false;
 }
 
+// whether the mbarrier's phase of the given parity is over, without waiting
+__device__ __forceinline__ bool mbar_test(uint64_t *mbar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred q;\n\tmbarrier.test_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(done) : "r"(smem_u32(mbar)), "r"(parity) : "memory");
+    return done != 0;
+}
+
 // TMEM allocation (one warp), address written to *dst (shared memory)
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst, uint32_t ncols)
 {
