@@ -35,6 +35,7 @@ struct akra_batch_s {
     int fft_mmax = 0;
     size_t fft_smem_set = 48 * 1024;     // dynamic shared memory the FFT kernel is cleared for
     akra::LegShape items_shape{0, 0, 0};
+    std::vector<unsigned> items_gens, titems_gens;   // the plans' weights the work lists were made for
     std::vector<int> nch;                 // Legendre chunks per instance (current shape)
     std::vector<char> blk;                // instances whose Legendre stages are block-jump launches of their own
     cudaGraphExec_t graph = nullptr;
@@ -67,18 +68,24 @@ static LegShape blk_shape(const LegShape &s)
     return t;
 }
 
-// (re)build the work-item lists for the batch's Legendre shape
+// the weights of every plan, which fix its ring pairs and rings
+static std::vector<unsigned> weights_gens(akra_batch b)
+{
+    std::vector<unsigned> g(b->ninst);
+    for (int i = 0; i < b->ninst; i++) g[i] = b->plans[i]->weights_gen;
+    return g;
+}
+
+// (re)build the work-item lists for the batch's Legendre shape and the plans' footprints
 static akra_status batch_items(akra_batch b)
 {
     const LegShape s = b->shape;
+    const std::vector<unsigned> gens = weights_gens(b);
+    if (b->items_gens == gens && s.P == b->items_shape.P && s.RG == b->items_shape.RG && s.NT == b->items_shape.NT)
+        return AKRA_OK;
+    b->items_gens.clear();   // set again once the lists are there
     std::vector<char> blk(b->ninst);
     for (int i = 0; i < b->ninst; i++) blk[i] = blk_pays(b->plans[i], b->plans[i]->d_active_units, true);
-    if (b->d_items && b->blk == blk)
-        for (int i = 0; i < b->ninst; i++)
-            if (blk[i])
-                b->nch[i] = legendre_chunks(b->plans[i], b->plans[i]->d_active_units, b->plans[i]->n_active_units, blk_shape(s));
-    if (b->d_items && b->blk == blk && s.P == b->items_shape.P && s.RG == b->items_shape.RG && s.NT == b->items_shape.NT)
-        return AKRA_OK;
     struct It { long long cost; int4 v; };
     std::vector<It> items;
     std::vector<int4> fitems;
@@ -119,13 +126,16 @@ static akra_status batch_items(akra_batch b)
     b->nitems = (int)hv.size();
     b->nfitems = (int)fitems.size();
     b->items_shape = s;
+    b->items_gens = gens;
     return AKRA_OK;
 }
 
 // (re)build the tensor-core synthesis items: (instance, m, 128-pair chunk, RHS group), heaviest first
 static akra_status batch_titems(akra_batch b)
 {
-    if (b->tcg == 0 || (b->d_titems && b->titems_tcg == b->tcg)) return AKRA_OK;
+    const std::vector<unsigned> gens = weights_gens(b);
+    if (b->tcg == 0 || (b->titems_gens == gens && b->titems_tcg == b->tcg)) return AKRA_OK;
+    b->titems_gens.clear();
     struct It { long long cost; int4 v; };
     std::vector<It> items;
     for (int i = 0; i < b->ninst; i++) {
@@ -152,6 +162,7 @@ static akra_status batch_titems(akra_batch b)
     AKRA_CUDA_TRY(cudaMemcpy(b->d_titems, hv.data(), sizeof(int4) * hv.size(), cudaMemcpyHostToDevice));
     b->ntitems = (int)hv.size();
     b->titems_tcg = b->tcg;
+    b->titems_gens = gens;
     return AKRA_OK;
 }
 

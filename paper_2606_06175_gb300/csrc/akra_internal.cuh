@@ -357,6 +357,7 @@ struct akra_plan_s {
     std::map<long long, akra::LegShape> shapes;   // key: prec*1000 + R
     std::map<long long, akra::CgGraph *> graphs;
     unsigned ws_gen = 0;                     // bumped whenever a workspace is reallocated
+    unsigned weights_gen = 0;                // bumped whenever the active ring and unit lists change
     const int *cur_skip = nullptr;           // device flag: operator kernels return early if set
     int *d_tc_err = nullptr;                 // device flag: a bounded wait inside a Legendre kernel ran out
     void *h_pinned = nullptr;                // pinned host mirror for status polling

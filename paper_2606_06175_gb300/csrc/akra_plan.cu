@@ -929,6 +929,7 @@ extern "C" akra_status akra_plan_set_weights(akra_plan p, const double *d_ninv, 
         if (one_ring[k]) steps_one += p->steps32[units[k]];
     }
     p->mostly_one_ring = steps_all > 0 && 2 * steps_one >= steps_all;
+    p->weights_gen++;
     AKRA_CUDA_TRY(cudaMemcpy(p->d_ring_active, active.data(), nr, cudaMemcpyHostToDevice));
     if (!rings.empty())
         AKRA_CUDA_TRY(cudaMemcpy(p->d_active_rings, rings.data(), sizeof(int) * rings.size(),
