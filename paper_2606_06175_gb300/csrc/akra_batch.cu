@@ -76,6 +76,13 @@ static std::vector<unsigned> weights_gens(akra_batch b)
     return g;
 }
 
+// a captured iteration holds the addresses and sizes of the work lists: dropped before a list is replaced
+static void drop_graph(akra_batch b)
+{
+    if (b->graph) cudaGraphExecDestroy(b->graph);
+    b->graph = nullptr;
+}
+
 // (re)build the work-item lists for the batch's Legendre shape and the plans' footprints
 static akra_status batch_items(akra_batch b)
 {
@@ -112,6 +119,7 @@ static akra_status batch_items(akra_batch b)
     std::stable_sort(items.begin(), items.end(), [](const It &a, const It &c) { return a.cost > c.cost; });
     std::vector<int4> hv(items.size());
     for (size_t k = 0; k < items.size(); k++) hv[k] = items[k].v;
+    drop_graph(b);
     if (b->d_items) cudaFree(b->d_items);
     if (b->d_fitems) cudaFree(b->d_fitems);
     b->d_items = b->d_fitems = nullptr;
@@ -152,6 +160,7 @@ static akra_status batch_titems(akra_batch b)
     std::stable_sort(items.begin(), items.end(), [](const It &a, const It &c) { return a.cost > c.cost; });
     std::vector<int4> hv(items.size());
     for (size_t k = 0; k < items.size(); k++) hv[k] = items[k].v;
+    drop_graph(b);
     if (b->d_titems) cudaFree(b->d_titems);
     b->d_titems = nullptr;
     if (cudaMalloc(&b->d_titems, sizeof(int4) * std::max<size_t>(hv.size(), 1)) != cudaSuccess) {
@@ -340,10 +349,7 @@ static bool graph_valid(akra_batch b)
 static akra_status batch_graph(akra_batch b, std::vector<CgBufs> &cb)
 {
     if (graph_valid(b)) return AKRA_OK;
-    if (b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+    drop_graph(b);
     std::vector<void *> xs(b->ninst), ys(b->ninst);
     std::vector<const int *> sk(b->ninst);
     for (int i = 0; i < b->ninst; i++) {
