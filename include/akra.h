@@ -149,7 +149,8 @@ akra_status akra_plan_fill_workspaces(akra_plan plan, int byte, void *stream);
  * and the list of rings with any nonzero weight (the only rings H needs).  An all-zero d_ninv
  * (empty footprint) is accepted: no ring is active, λ_eff = 0, H = 0 and solves return x = 0.
  * Blocking (reads the statistics back).  Errors: EINVAL (NULL, lambda < 0, negative or
- * non-finite N^-1), ECUDA. */
+ * non-finite N^-1), ENOMEM, ECUDA.  NULL and lambda < 0 leave the plan as it was; after any other
+ * failure it has no weights (ENOWEIGHTS) until a call succeeds. */
 akra_status akra_plan_set_weights(akra_plan plan, const double *d_ninv, double lambda,
                                   void *stream);
 

@@ -178,6 +178,11 @@ static akra_status batch_titems(akra_batch b)
 // FP32 workspaces of every instance for the batch shape, and FP64 ones for the outer residual
 static akra_status batch_reserve(akra_batch b)
 {
+    for (int i = 0; i < b->ninst; i++)
+        if (!b->plans[i]->has_weights) {
+            set_error("akra_batch: the last akra_plan_set_weights of plan %d failed", i);
+            return AKRA_ENOWEIGHTS;
+        }
     AKRA_TRY(batch_items(b));
     AKRA_TRY(batch_titems(b));
     for (int i = 0; i < b->ninst; i++) {

@@ -608,6 +608,8 @@ akra_status flat_set_weights(akra_plan p, const double *d_ninv, double lambda, c
         return AKRA_ENOMEM;
     }
     double h[3] = {0, 0, 0};
+    p->has_weights = false;   // until the new ones are complete
+    p->ws_gen++;   // captured CG iterations hold the previous λ_eff
     cudaError_t e = cudaMemsetAsync(d_stats, 0, 3 * sizeof(double), st);
     if (e == cudaSuccess) {
         flat::k_weights<<<1216, 256, 0, st>>>(p->nside, d_ninv, p->d_W64, p->d_W32, p->d_fWt64, p->d_fWt32, d_stats);
@@ -627,7 +629,6 @@ akra_status flat_set_weights(akra_plan p, const double *d_ninv, double lambda, c
     p->precond = 1.0 / (h[0] / (double)p->npix + p->lambda_eff);
     if (!std::isfinite(p->precond)) p->precond = 1.0;
     p->has_weights = true;
-    p->ws_gen++;   // captured CG iterations hold the previous λ_eff
     return AKRA_OK;
 }
 

@@ -197,7 +197,6 @@ struct BlkTables {
     BlkChunk *info = nullptr;
     uint4 *vtab = nullptr;
     int nrows = 0, nchunks = 0, npolar = 0;
-    size_t cap_rows = 0;
 };
 
 // smallest band limit at which the block-jump kernels run (their smallest measured gain: 64 / 128)
@@ -390,6 +389,7 @@ akra_status legendre_synth_tc_queue(int tcg, const LegArgs<float> *insts, const 
                                     int *counter, cudaStream_t st);
 // block-jump Legendre kernels (akra_legendre_blk.cu); rows: the ring rows of the list, ascending, and
 // npolar how many of its ring pairs lie within 0.1 rad of a pole
+akra_status blk_tables_alloc(akra_plan p, BlkTables &t);
 akra_status blk_tables_build(akra_plan p, BlkTables &t, const std::vector<int> &rows, int npolar, cudaStream_t st);
 void blk_tables_free(BlkTables &t);
 akra_status legendre_blk_prepare();

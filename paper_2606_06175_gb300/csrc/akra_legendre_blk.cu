@@ -151,22 +151,25 @@ void blk_tables_free(BlkTables &t)
     t = BlkTables();
 }
 
+// tables that hold any ring list of the plan (at plan creation, so that new weights allocate nothing)
+akra_status blk_tables_alloc(akra_plan p, BlkTables &t)
+{
+    const size_t cap = p->nring, cch = (cap + BLK_RINGS - 1) / BLK_RINGS;
+    const size_t bytes[3] = {sizeof(int) * cap, sizeof(BlkChunk) * cch, BLK_VBYTES * cch};
+    if (cudaMalloc((void **)&t.rows, bytes[0]) != cudaSuccess || cudaMalloc((void **)&t.info, bytes[1]) != cudaSuccess ||
+        cudaMalloc((void **)&t.vtab, bytes[2]) != cudaSuccess) {
+        cudaGetLastError();
+        blk_tables_free(t);
+        set_error("plan table allocation failed");
+        return AKRA_ENOMEM;
+    }
+    p->bytes_tables += bytes[0] + bytes[1] + bytes[2];
+    return AKRA_OK;
+}
+
 akra_status blk_tables_build(akra_plan p, BlkTables &t, const std::vector<int> &rows, int npolar, cudaStream_t st)
 {
     const int n = (int)rows.size(), nch = (n + BLK_RINGS - 1) / BLK_RINGS;
-    if (rows.size() > t.cap_rows) {
-        const size_t cap = p->nring, cch = (cap + BLK_RINGS - 1) / BLK_RINGS;   // every list fits from now on
-        const size_t bytes[3] = {sizeof(int) * cap, sizeof(BlkChunk) * cch, BLK_VBYTES * cch};
-        if (cudaMalloc((void **)&t.rows, bytes[0]) != cudaSuccess || cudaMalloc((void **)&t.info, bytes[1]) != cudaSuccess ||
-            cudaMalloc((void **)&t.vtab, bytes[2]) != cudaSuccess) {
-            cudaGetLastError();
-            blk_tables_free(t);
-            set_error("plan table allocation failed");
-            return AKRA_ENOMEM;
-        }
-        p->bytes_tables += bytes[0] + bytes[1] + bytes[2];
-        t.cap_rows = cap;
-    }
     t.nrows = n;
     t.nchunks = nch;
     t.npolar = npolar;

@@ -690,6 +690,8 @@ static akra_status plan_build(akra_plan p)
     AKRA_TRY(ring_fft32_build(p));
     AKRA_TRY(legendre_tc_prepare());
     AKRA_TRY(legendre_blk_prepare());
+    AKRA_TRY(blk_tables_alloc(p, p->blk_all));
+    AKRA_TRY(blk_tables_alloc(p, p->blk_act));
     {
         std::vector<int> rings(p->nring);
         for (int r = 0; r < p->nring; r++) rings[r] = r;
@@ -881,6 +883,9 @@ extern "C" akra_status akra_plan_set_weights(akra_plan p, const double *d_ninv, 
         set_error("akra_plan_set_weights: scratch allocation failed");
         return AKRA_ENOMEM;
     }
+    // from here until everything that goes with the new weights is there the plan has none
+    p->has_weights = false;
+    p->ws_gen++;   // captured CG iterations hold the previous active lists and λ_eff
     k_weights<<<nr, 256, 0, st>>>(p->d_rings, d_ninv, p->omega, p->d_W64, p->d_W32, p->d_W32r, d_stats,
                                   d_stats + nr, d_stats + 2 * nr);
     std::vector<double> h(3 * (size_t)nr);
@@ -949,11 +954,11 @@ extern "C" akra_status akra_plan_set_weights(akra_plan p, const double *d_ninv, 
                                       p->d_pw32);
     AKRA_CUDA_TRY(cudaGetLastError());
     AKRA_CUDA_TRY(cudaStreamSynchronize(st));
-    p->has_weights = true;
-    p->ws_gen++;   // captured CG iterations hold the previous active lists and λ_eff
     AKRA_TRY(blk_build(p, p->blk_act, rings, st));
     AKRA_CUDA_TRY(cudaStreamSynchronize(st));   // later calls may come on other streams
-    return ring_fft32_order(p, rings, p->d_fft32_rings_act, &p->fft32_nsmall_act);
+    AKRA_TRY(ring_fft32_order(p, rings, p->d_fft32_rings_act, &p->fft32_nsmall_act));
+    p->has_weights = true;
+    return AKRA_OK;
 }
 
 static akra_status check_common(akra_plan p, akra_prec prec, const void *a, const void *b, int R,
