@@ -405,6 +405,8 @@ akra_status tc_error_check(akra_plan p);
 
 LegShape leg_shape(akra_plan p, akra_prec prec, int R);
 int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s);
+int adjoint_rhs(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);
+size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);
 void cg_release_graphs(akra_plan p);   // akra_cg.cu
 akra_status metric_inverse(akra_plan p, bool dbl, const void *in, void *out, int R, cudaStream_t st);
 
@@ -427,6 +429,23 @@ template <typename T>
 akra_status adjoint_epilogue(akra_plan p, LegMode mode, const void *partial, int nchunks,
                              const void *x_reg, double lam, void *alm_out, int R, cudaStream_t st,
                              int fields = 3);
+
+// the adjoint of R right-hand sides, adjoint_rhs of them at a time; then(r, n, nchunks) finishes those from r to
+// r + n - 1, whose partial sums the next ones overwrite
+template <typename T, typename F>
+akra_status legendre_adjoint_groups(akra_plan p, const LegShape &s, const void *phi, void *partial, int R,
+                                    const int *units, int nunits, cudaStream_t st, F &&then)
+{
+    const int g = adjoint_rhs(p, units, nunits, s, R, sizeof(T));
+    const size_t per = (size_t)p->nring * (2 * (size_t)p->lmax + 1);
+    for (int r = 0; r < R; r += g) {
+        const int n = R - r < g ? R - r : g;
+        int nch = 0;
+        AKRA_TRY(legendre_adjoint<T>(p, s, (const cx_t<T> *)phi + r * per, partial, n, units, nunits, &nch, st));
+        AKRA_TRY(then(r, n, nch));
+    }
+    return AKRA_OK;
+}
 
 enum class FftMode { Synth = 0, Adjoint = 1, Happly = 2 };
 template <typename T>

@@ -272,6 +272,27 @@ int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s
     return (nunits + per - 1) / per;
 }
 
+// Right-hand sides whose partial sums are formed at a time.  Chunks of 256 rings have about twice the partial
+// sums of the direct kernel's 640 pairs: 12 chunks against 5 on the DES-like footprint at Nside 2048 / lmax 4096, 1.6 GB
+// per right-hand side against 0.67, 103 GB against 43 at 64.  They take no more than the direct kernel's, or 4 GB (where
+// launches of a millisecond and more are split, which costs nothing that can be measured), so that a call that
+// fits with the direct kernel fits with these.
+int adjoint_rhs(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes)
+{
+    if (!s.BA || nunits <= 0 || !blk_pays(p, units, true)) return R;
+    const size_t vec = (size_t)p->ntri * 4 * real_bytes;
+    const size_t most = std::max((size_t)((nunits + 639) / 640) * R * vec, (size_t)4 << 30);
+    const size_t fit = std::max<size_t>(most / (vec * legendre_chunks(p, units, nunits, s)), 1);
+    if (fit >= (size_t)R) return R;
+    const int groups = (int)((R + fit - 1) / fit);
+    return (R + groups - 1) / groups;   // of even size
+}
+
+size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes)
+{
+    return (size_t)legendre_chunks(p, units, nunits, s) * adjoint_rhs(p, units, nunits, s, R, real_bytes) * p->ntri * 4 * real_bytes;
+}
+
 template LegArgs<float> leg_args<float>(akra_plan, const LegShape &, LegMode, const int *, int, int);
 template LegArgs<double> leg_args<double>(akra_plan, const LegShape &, LegMode, const int *, int, int);
 template akra_status legendre_synth<float>(akra_plan, const LegShape &, LegMode, const void *, void *,

@@ -525,12 +525,11 @@ akra_status op_adjoint(akra_plan p, LegMode mode, const void *map, void *alm, bo
     const int *rings = act ? p->d_active_rings : p->d_all_rings;
     const int nrings = act ? p->n_active_rings : p->nring;
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
-    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(p, units, nunits, s) * R * p->ntri * 4 *
-                                           sizeof(T)));
+    AKRA_TRY(ws_reserve(p, p->partial, partial_bytes(p, units, nunits, s, R, sizeof(T))));
     AKRA_TRY(ring_fft<T>(p, FftMode::Adjoint, p->phi.ptr, map, nullptr, weighted, R, rings, nrings, st));
-    int nch = 0;
-    AKRA_TRY(legendre_adjoint<T>(p, s, p->phi.ptr, p->partial.ptr, R, units, nunits, &nch, st));
-    return adjoint_epilogue<T>(p, mode, p->partial.ptr, nch, nullptr, 0.0, alm, R, st);
+    return legendre_adjoint_groups<T>(p, s, p->phi.ptr, p->partial.ptr, R, units, nunits, st, [&](int r, int n, int nch) {
+        return adjoint_epilogue<T>(p, mode, p->partial.ptr, nch, nullptr, 0.0, (cx_t<T> *)alm + (size_t)r * 2 * p->ntri, n, st);
+    });
 }
 
 template <typename T>
@@ -539,17 +538,17 @@ akra_status op_H(akra_plan p, const void *x, void *y, int R, cudaStream_t st)
     if (is_flat(p)) return flat_op_H<T>(p, x, y, R, st);
     const LegShape s = leg_shape(p, prec_of<T>(), R);
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
-    AKRA_TRY(ws_reserve(p, p->partial, (size_t)legendre_chunks(p, p->d_active_units, p->n_active_units, s) * R *
-                                           p->ntri * 4 * sizeof(T)));
+    AKRA_TRY(ws_reserve(p, p->partial, partial_bytes(p, p->d_active_units, p->n_active_units, s, R, sizeof(T))));
     AKRA_TRY(legendre_synth<T>(p, s, LegMode::KS, x, p->phi.ptr, R, p->d_active_units,
                                p->n_active_units, st));
     AKRA_TRY(ring_fft<T>(p, FftMode::Happly, p->phi.ptr, nullptr, nullptr, true, R,
                          p->d_active_rings, p->n_active_rings, st));
-    int nch = 0;
-    AKRA_TRY(legendre_adjoint<T>(p, s, p->phi.ptr, p->partial.ptr, R, p->d_active_units,
-                                 p->n_active_units, &nch, st));
-    return adjoint_epilogue<T>(p, LegMode::KS, p->partial.ptr, nch, x, p->lambda_eff, y, R, st,
-                               p->fields);
+    return legendre_adjoint_groups<T>(p, s, p->phi.ptr, p->partial.ptr, R, p->d_active_units, p->n_active_units, st,
+                                      [&](int r, int n, int nch) {
+        const size_t at = (size_t)r * 2 * p->ntri;
+        return adjoint_epilogue<T>(p, LegMode::KS, p->partial.ptr, nch, (const cx_t<T> *)x + at, p->lambda_eff,
+                                   (cx_t<T> *)y + at, n, st, p->fields);
+    });
 }
 
 template akra_status op_synth<float>(akra_plan, LegMode, const void *, void *, bool, int, cudaStream_t);
@@ -1072,7 +1071,7 @@ static akra_status tune_one(akra_plan p, akra_prec prec, int R, cudaStream_t st)
     }
     size_t max_part = 0;
     for (auto &c : cands)
-        max_part = std::max(max_part, (size_t)legendre_chunks(p, units, nunits, c) * (size_t)R * (size_t)p->ntri * 4 * sizeof(T));
+        max_part = std::max(max_part, partial_bytes(p, units, nunits, c, R, sizeof(T)));
     AKRA_TRY(ws_reserve(p, p->phi, (size_t)R * p->nring * (2 * (size_t)p->lmax + 1) * sizeof(cx_t<T>)));
     AKRA_TRY(ws_reserve(p, p->partial, max_part));
     void *alm = nullptr;
@@ -1093,11 +1092,12 @@ static akra_status tune_one(akra_plan p, akra_prec prec, int R, cudaStream_t st)
     for (size_t k = 0; k < cands.size() && s == AKRA_OK; k++) {
         const LegShape &c = cands[k];
         for (int rep = 0; rep < 3 && s == AKRA_OK; rep++) {
-            int nch = 0;
             cudaEventRecord(e0, st);
             s = legendre_synth<T>(p, c, LegMode::KS, alm, p->phi.ptr, R, units, nunits, st);
             cudaEventRecord(e1, st);
-            if (s == AKRA_OK) s = legendre_adjoint<T>(p, c, p->phi.ptr, p->partial.ptr, R, units, nunits, &nch, st);
+            if (s == AKRA_OK)
+                s = legendre_adjoint_groups<T>(p, c, p->phi.ptr, p->partial.ptr, R, units, nunits, st,
+                                               [](int, int, int) { return AKRA_OK; });
             cudaEventRecord(e2, st);
             cudaEventSynchronize(e2);
             float m1 = 0, m2 = 0;
@@ -1274,9 +1274,8 @@ static akra_status time_stages(akra_plan p, int R, int reps, cudaStream_t st, do
 {
     const akra_prec prec = prec_of<T>();
     const LegShape s = leg_shape(p, prec, R);
-    const int nch = legendre_chunks(p, p->d_active_units, p->n_active_units, s);
     AKRA_TRY(ws_reserve(p, p->phi, phi_bytes(p, sizeof(cx_t<T>), R)));
-    AKRA_TRY(ws_reserve(p, p->partial, (size_t)nch * R * p->ntri * 4 * sizeof(T)));
+    AKRA_TRY(ws_reserve(p, p->partial, partial_bytes(p, p->d_active_units, p->n_active_units, s, R, sizeof(T))));
     void *x = nullptr, *y = nullptr;
     const size_t ab = (size_t)R * 2 * p->ntri * sizeof(cx_t<T>);
     if (cudaMalloc(&x, ab) != cudaSuccess || cudaMalloc(&y, ab) != cudaSuccess) {
@@ -1291,7 +1290,7 @@ static akra_status time_stages(akra_plan p, int R, int reps, cudaStream_t st, do
     double acc[5] = {0, 0, 0, 0, 0};
     akra_status s1 = AKRA_OK;
     for (int rep = 0; rep <= reps && s1 == AKRA_OK; rep++) {
-        int n2 = 0;
+        int g = 1, n2 = 0;
         cudaEventRecord(ev[0], st);
         s1 = legendre_synth<T>(p, s, LegMode::KS, x, p->phi.ptr, R, p->d_active_units, p->n_active_units, st);
         cudaEventRecord(ev[1], st);
@@ -1300,10 +1299,16 @@ static akra_status time_stages(akra_plan p, int R, int reps, cudaStream_t st, do
                              p->n_active_rings, st);
         cudaEventRecord(ev[2], st);
         if (s1 == AKRA_OK)
-            s1 = legendre_adjoint<T>(p, s, p->phi.ptr, p->partial.ptr, R, p->d_active_units,
-                                     p->n_active_units, &n2, st);
+            s1 = legendre_adjoint_groups<T>(p, s, p->phi.ptr, p->partial.ptr, R, p->d_active_units, p->n_active_units, st,
+                                            [&](int r, int n, int nch) {
+                g = r == 0 ? n : g;   // the largest group
+                n2 = nch;
+                return AKRA_OK;
+            });
         cudaEventRecord(ev[3], st);
-        if (s1 == AKRA_OK) s1 = adjoint_epilogue<T>(p, LegMode::KS, p->partial.ptr, n2, x, p->lambda_eff, y, R, st);
+        for (int r = 0; r < R && s1 == AKRA_OK; r += g)   // each on the last group's sums
+            s1 = adjoint_epilogue<T>(p, LegMode::KS, p->partial.ptr, n2, (const cx_t<T> *)x + (size_t)r * 2 * p->ntri,
+                                     p->lambda_eff, (cx_t<T> *)y + (size_t)r * 2 * p->ntri, std::min(g, R - r), st);
         cudaEventRecord(ev[4], st);
         cudaEventSynchronize(ev[4]);
         if (rep == 0) continue;   // warm-up
