@@ -387,8 +387,8 @@ akra_status akra_plan_get_adjoint_shape(akra_plan plan, akra_prec prec, int R, i
  * the recurrences stay on the CUDA cores, their values split into a TF32 head and an FP32
  * remainder, and the l-sum is three TF32 products (head·head, head·rest, rest·head) accumulated in
  * FP32 -- about 21 bits per product, within the FP32 operator's tolerance.  Groups of 4 and 8, on
- * footprints of one hemisphere (lmax >= 128), run the block-jump kernel that group = 0 runs
- * there, which is faster (unless akra_plan_set_shape has fixed the shape).  group = 0 selects the
+ * footprints of one hemisphere (lmax >= 128), run the kernel that group = 0 runs there, which
+ * is faster (unless akra_plan_set_shape has fixed the shape).  group = 0 selects the
  * CUDA-core synthesis.  akra_autotune considers both; akra_plan_set_shape resets the choice to
  * the CUDA-core synthesis.  If a tensor-core completion wait exceeds its bound (it should not),
  * the next blocking call (a solve, akra_autotune, akra_time_H_stages) returns ECUDA.

@@ -63,7 +63,7 @@ static int num_sms()
 static LegShape blk_shape(const LegShape &s)
 {
     LegShape t = s;
-    t.BS = t.BA = 1;
+    t.BS = t.BA = 2;
     t.TC = 0;
     return t;
 }

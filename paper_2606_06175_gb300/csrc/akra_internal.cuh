@@ -178,7 +178,8 @@ struct LegShape {
     int TC = 0;            // FP32 synthesis on the tensor core with RHS groups of TC (4, 8, 16,
                            // 32); 0: CUDA-core synthesis of shape (P, RG)
     int RGA = 0;           // RHS per block of the adjoint (0: same as RG)
-    int BS = 0, BA = 0;    // FP32 synthesis / adjoint by 16-step block jumps (akra_legendre_blk.cuh)
+    int BS = 0, BA = 0;    // FP32 synthesis / adjoint by 16-step block jumps (akra_legendre_blk.cuh) on lists of
+                           // blk_pays: 1 where that is measured faster (jump_synth, adjoint_shape), 2 always
     int adjP() const { return PA > 0 ? PA : P; }
     int adjRG() const { return RGA > 0 ? RGA : RG; }
 };
@@ -405,6 +406,7 @@ akra_status tc_error_check(akra_plan p);
 
 LegShape leg_shape(akra_plan p, akra_prec prec, int R);
 int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s);
+LegShape adjoint_shape(akra_plan p, const LegShape &s, const int *units, int nunits, int R);
 int adjoint_rhs(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);
 size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);
 void cg_release_graphs(akra_plan p);   // akra_cg.cu
@@ -433,9 +435,10 @@ akra_status adjoint_epilogue(akra_plan p, LegMode mode, const void *partial, int
 // the adjoint of R right-hand sides, adjoint_rhs of them at a time; then(r, n, nchunks) finishes those from r to
 // r + n - 1, whose partial sums the next ones overwrite
 template <typename T, typename F>
-akra_status legendre_adjoint_groups(akra_plan p, const LegShape &s, const void *phi, void *partial, int R,
+akra_status legendre_adjoint_groups(akra_plan p, const LegShape &shape, const void *phi, void *partial, int R,
                                     const int *units, int nunits, cudaStream_t st, F &&then)
 {
+    const LegShape s = adjoint_shape(p, shape, units, nunits, R);   // of all R, whatever the groups
     const int g = adjoint_rhs(p, units, nunits, s, R, sizeof(T));
     const size_t per = (size_t)p->nring * (2 * (size_t)p->lmax + 1);
     for (int r = 0; r < R; r += g) {

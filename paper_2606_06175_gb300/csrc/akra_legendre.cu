@@ -157,6 +157,52 @@ bool blk_pays(akra_plan p, const int *units, bool adjoint)
     return !adjoint && p->lmax >= 4096;
 }
 
+// Synthesis of R right-hand sides on a list of blk_pays.  A block-jump block takes one right-hand side, a direct
+// block of shape (1, 4) four that share the recurrence, so from four on the direct kernel is the faster one where its
+// slots are full and lmax is low.  Time of (1, 4) over block jumps at full slots (R = 4, 8) on DES-like footprints: 256 / 512
+// 0.66, 300 / 600 0.78, 512 / 1024 1.01, 1024 / 1024 1.04, 1024 / 2048 1.25; caps 0.63, 0.63, 0.84, 0.85, 1.00; about 0.62 + 0.3 lmax / 1000
+// between them, more by the empty slots (R = 5 at 400 / 800: 1.18 to 1.32).  One to three right-hand sides: 1.18 to 1.97 with
+// one, 0.9 to 1.35 with two or three (below 1 at a few sizes of lmax 250 to 800 only, and the block jumps are the
+// more accurate ones).  All rings, 2048 / 4096: R = 1 1.14, 2 1.08, 3 1.16, 4 0.94, 6 1.09.
+static bool jump_synth(akra_plan p, const LegShape &s, const int *units, int R)
+{
+    if (!s.BS || !blk_pays(p, units, false)) return false;
+    if (s.BS == 2 || R < 4) return true;
+    const double pad = (R + 3) / 4 * 4 / (double)R;
+    return units == p->d_all_units ? pad >= 1.06 : pad * (0.62 + 0.3e-3 * p->lmax) >= 0.95;
+}
+
+// The adjoint's shape on a list of blk_pays: whether the block jumps take it (BA 2 or 0), for all of R, and the direct
+// shape where they do not.  The block jumps repeat for every right-hand side what a direct block does once (seeds, staging,
+// the warp reduction's set-up), compute the rings that pad a chunk, and pay a set-up, a slow first phase and a padded last
+// tile per block, for short l-ranges of many chunks above all.  Adjoint and epilogue in us, direct, block jumps (footprints:
+// DES-like; 30-degree cap):
+//   R = 1: 128 / 256 31, 24; 31, 26; 400 / 800 156, 158; 120, 124; 600 / 1200 376, 396; 288, 324; 1024 / 1024 399, 458; 349, 420; 2048 / 4096
+//          9857, 9172; 7316, 7465: the block jumps, whose errors are smaller by up to a third, but where lmax is below
+//          Nside (1500 / 1024 566, 668; 424, 558; 2048 / 1024 724, 878; 573, 749) and on a strip that fills its chunks badly (400 / 800,
+//          559 rings 125, 158)
+//   R = 2: 128 / 256 37, 35; 37, 35; 200 / 250 39, 45; 40, 36 (one chunk); 300 / 600 125, 143; 115, 140; 600 / 700 278, 323; 220, 260
+//   R = 5: 64 / 128 24, 30; 22, 30; 200 / 250 62, 92; 56, 63; 400 / 800 648, 743; 455, 566; 600 / 1200 1789, 1934; 1285, 1551
+//   R = 8: 400 / 400 296, 399; 221, 297; 1024 / 1024 3060, 3540; 2520, 3230; 1024 / 2048 11400, 11404; 9200, 10183
+// The direct shape is the one with the fewest pairs of padding: a single chunk up to 640 pairs, chunks of 384 or 512
+// beyond (400 / 800 with R = 5, 555 pairs: (5, 1) 648, (3, 1) 612, (4, 1) 728; 200 / 400, 278 pairs: (3, 1) 113, (2, 1) 139, (5, 1) 181).
+LegShape adjoint_shape(akra_plan p, const LegShape &s, const int *units, int nunits, int R)
+{
+    LegShape t = s;
+    if (s.BA != 1 || nunits <= 0 || !blk_pays(p, units, true)) return t;
+    const BlkTables &bt = blk_tables(p, units);
+    const bool badly_filled = bt.nrows < 0.8 * 256 * bt.nchunks;
+    bool direct = bt.nchunks >= 3 && p->lmax < p->nside;
+    if (R >= 3 || (R == 2 && bt.nchunks >= 2)) direct |= p->lmax < 1100 || badly_filled;
+    if (R == 1 && bt.nchunks >= 2) direct |= badly_filled && p->one_side != 0 && p->nside * (double)p->lmax >= 2.2e5;
+    t.BA = direct ? 0 : 2;
+    if (!direct) return t;
+    const int c = (nunits + 127) / 128;
+    t.PA = c <= 5 ? c : (c + 3) / 4 * 4 <= (c + 2) / 3 * 3 ? 4 : 3;
+    t.RGA = 1;
+    return t;
+}
+
 // shape dispatch: (P, RG) combinations compiled for each precision, NT = 128
 template <typename T>
 akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const void *alm,
@@ -164,14 +210,13 @@ akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const v
 {
     if (nunits <= 0) return AKRA_OK;
     if constexpr (std::is_same<T, float>::value) {
-        // Groups of 4 and 8 RHS leave the tensor-core GEMM's columns thin: on one-ring lists the block-jump kernel,
-        // whose own contractions are on the tensor cores, takes them too.  Synthesis, ms, groups -> block jumps:
-        // (1024, 2048) 8 RHS of 4 12.7, of 8 9.17 -> 5.42; (512, 1024) 1.79, 1.32 -> 0.95.  16 RHS of 16 10.3
-        // against 10.8 and 1.55 against 1.89: larger groups stay.
-        const bool jump = s.BS && blk_pays(p, units, false);
-        if (s.TC > 0 && !(jump && s.TC <= 8 && blk_pays(p, units, true)))
+        // Groups of 4 and 8 RHS leave the tensor-core GEMM's columns thin: on one-ring lists what the default runs there
+        // is faster.  Synthesis of 8 RHS in us, groups of 4, of 8, the default: (128, 256) 65, 55, 34; (300, 600) 465,
+        // 357, 228 (direct); (1024, 2048) 12700, 9160, 5400 (block jumps).  Larger groups stay: 16 RHS of 16 10.3 ms
+        // against 10.8 at (1024, 2048).
+        if (s.TC > 0 && !(s.BS && s.TC <= 8 && blk_pays(p, units, true)))
             return legendre_synth_tc(p, s.TC, mode, alm, phi, R, units, nunits, st);
-        if (jump) {
+        if (jump_synth(p, s, units, R)) {
             // the polar ring pairs (the first of the list) keep the difference-form kernels
             const int npolar = blk_tables(p, units).npolar;
             LegShape sp = s;
@@ -288,8 +333,9 @@ int adjoint_rhs(akra_plan p, const int *units, int nunits, const LegShape &s, in
     return (R + groups - 1) / groups;   // of even size
 }
 
-size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes)
+size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &shape, int R, size_t real_bytes)
 {
+    const LegShape s = adjoint_shape(p, shape, units, nunits, R);
     return (size_t)legendre_chunks(p, units, nunits, s) * adjoint_rhs(p, units, nunits, s, R, real_bytes) * p->ntri * 4 * real_bytes;
 }
 

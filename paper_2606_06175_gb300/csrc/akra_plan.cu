@@ -457,11 +457,13 @@ LegShape leg_shape(akra_plan p, akra_prec prec, int R)
     //   FP64  W = 0.4 (32/64) (1,1) 39 (4,1) 86; W = 13 (128/256) (1,1) 301 (2,1) 289 (4,1) 447;
     //         W = 54 (256/512) (2,1) 1083 (4,1) 1087; R = 4: W = 30 (2,1) 444 (2,2) 462, W = 54 (2,1) 665
     //         (2,2) 539; synthesis R = 4: W = 14 (1,1) 97 (1,4) 167, W = 54 (1,2) 345 (1,4) 389, W = 216
-    //         (1,2) 2118 (1,4) 1817
+    //         (1,2) 2118 (1,4) 1817; synthesis R = 2, full sky and DES-like: W = 7 (1,1) 97, 70 (1,2) 95, 95; W = 15 223, 158
+    //         and 245, 155; W = 27 389, 263 and 416, 255; W = 50 846, 479 and 674, 376; R = 3 W = 10 126, 85 and 156, 111
     //   FP32 (full sky; the block-jump kernels take the lists of blk_pays)  W = 10 (96/251) (1,1) 41 (2,1) 53
     //         (5,1) 94; W = 121 (384/768) (2,1) 238 (3,1) 244 (5,1) 399; W = 403 (700/1400) (2,1) 1097 (3,1) 986
     //         (5,1) 1541; W = 863 (1024/2048) (3,1) 2645 (4,1) 2567 (5,1) 3475; R = 4: W = 216 (2,1) 311 (2,2)
-    //         274 (5,1) 533
+    //         274 (5,1) 533; odd R leaves a slot of (2,2) empty: R = 3 W = 41 (2,1) 67 (2,2) 74, W = 162 249, 273, W = 647
+    //         1344, 1637; R = 5 W = 1358 2977, 3340; even: R = 6 W = 324 (2,1) 448 (2,2) 413
     const double W = 2.0 * p->nside * (p->lmax + 1.0) * R / (32.0 * 152.0);
     if (prec == AKRA_F64) {
         LegShape s{1, 128, R >= 4 && W >= 100 ? 4 : R >= 2 && W >= 20 ? 2 : 1};
@@ -470,22 +472,14 @@ LegShape leg_shape(akra_plan p, akra_prec prec, int R)
         return s;
     }
     LegShape s{1, 128, R >= 4 ? 4 : R >= 2 ? 2 : 1};
-    if (R >= 2 && W >= 40 && W < 1500) s.PA = s.RGA = 2;
-    else {
+    if (R >= 2 && W >= 40 && W < 1500) {
+        s.PA = 2;
+        s.RGA = R % 2 == 0 || R >= 9 ? 2 : 1;
+    } else {
         s.PA = W < 16 ? 1 : W < 150 ? 2 : W < 600 ? 3 : 4;
         s.RGA = 1;
     }
-    s.BS = s.BA = 1;   // the block-jump kernels where they pay (blk_pays)
-    // From 3 RHS on a footprint that fills its chunks badly stays with the direct adjoint, at 5 pairs and one RHS
-    // per block.  A^T, direct -> block jumps, us, 5 RHS: 548 rings in 3 chunks (71 %; Nside 400) lmax 500
-    // 454 -> 493, lmax 800 839 -> 883 (880 at 2 pairs and 2 RHS); 822 in 4 (80 %; 600) lmax 700 1291 -> 1217, lmax
-    // 1200 2704 -> 2340; 351 in 2 (69 %; 256) 183 -> 168, few enough for its latency to count.
-    const BlkTables &t = p->blk_act;
-    if (R >= 3 && p->mostly_one_ring && t.nchunks >= 3 && t.nrows < 0.77 * 256 * t.nchunks) {
-        s.BA = 0;
-        s.PA = 5;
-        s.RGA = 1;
-    }
+    s.BS = s.BA = 1;   // the block-jump kernels where they pay (jump_synth, adjoint_shape)
     return s;
 }
 
@@ -1065,8 +1059,8 @@ static akra_status tune_one(akra_plan p, akra_prec prec, int R, cudaStream_t st)
     // FP32: the block-jump kernels, tried first (equal times keep them)
     if (std::is_same<T, float>::value && blk_pays(p, units, false)) {
         LegShape c{1, 128, 1, 5, 0, 1};
-        c.BS = 1;
-        c.BA = blk_pays(p, units, true);
+        c.BS = 2;
+        c.BA = blk_pays(p, units, true) ? 2 : 0;
         cands.insert(cands.begin(), c);
     }
     size_t max_part = 0;
