@@ -406,6 +406,7 @@ akra_status tc_error_check(akra_plan p);
 
 LegShape leg_shape(akra_plan p, akra_prec prec, int R);
 int legendre_chunks(akra_plan p, const int *units, int nunits, const LegShape &s);
+int synth_tc_group(akra_plan p, const LegShape &s, const int *units);
 LegShape adjoint_shape(akra_plan p, const LegShape &s, const int *units, int nunits, int R);
 int adjoint_rhs(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);
 size_t partial_bytes(akra_plan p, const int *units, int nunits, const LegShape &s, int R, size_t real_bytes);

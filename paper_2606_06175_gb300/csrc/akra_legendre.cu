@@ -203,6 +203,15 @@ LegShape adjoint_shape(akra_plan p, const LegShape &s, const int *units, int nun
     return t;
 }
 
+// The tensor-core group that a synthesis of shape s runs with (0: none).  Groups of 4 and 8 RHS leave the tensor-core
+// GEMM's columns thin: on one-ring lists what the default runs there is faster.  Synthesis of 8 RHS in us, groups of
+// 4, of 8, the default: (128, 256) 65, 55, 34; (300, 600) 465, 357, 228 (direct); (1024, 2048) 12700, 9160, 5400 (block
+// jumps).  Larger groups stay: 16 RHS of 16 10.3 ms against 10.8 at (1024, 2048).
+int synth_tc_group(akra_plan p, const LegShape &s, const int *units)
+{
+    return s.BS && s.TC <= 8 && blk_pays(p, units, true) ? 0 : s.TC;
+}
+
 // shape dispatch: (P, RG) combinations compiled for each precision, NT = 128
 template <typename T>
 akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const void *alm,
@@ -210,12 +219,8 @@ akra_status legendre_synth(akra_plan p, const LegShape &s, LegMode mode, const v
 {
     if (nunits <= 0) return AKRA_OK;
     if constexpr (std::is_same<T, float>::value) {
-        // Groups of 4 and 8 RHS leave the tensor-core GEMM's columns thin: on one-ring lists what the default runs there
-        // is faster.  Synthesis of 8 RHS in us, groups of 4, of 8, the default: (128, 256) 65, 55, 34; (300, 600) 465,
-        // 357, 228 (direct); (1024, 2048) 12700, 9160, 5400 (block jumps).  Larger groups stay: 16 RHS of 16 10.3 ms
-        // against 10.8 at (1024, 2048).
-        if (s.TC > 0 && !(s.BS && s.TC <= 8 && blk_pays(p, units, true)))
-            return legendre_synth_tc(p, s.TC, mode, alm, phi, R, units, nunits, st);
+        const int tcg = synth_tc_group(p, s, units);
+        if (tcg > 0) return legendre_synth_tc(p, tcg, mode, alm, phi, R, units, nunits, st);
         if (jump_synth(p, s, units, R)) {
             // the polar ring pairs (the first of the list) keep the difference-form kernels
             const int npolar = blk_tables(p, units).npolar;
