@@ -123,9 +123,8 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_synth_blk(LegArgs<float>
     if (a.skip && *a.skip) return;
     const uint32_t tmem = blk_open(&s_tmem, &bars);
     const int m = blockIdx.x / a.blk_chunks;
-    uint32_t tiles = 0;
-    blk_synth_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tiles, tmem);
-    blk_close<false>(tmem, &bars, (int)tiles);
+    const int T = blk_synth_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tmem);
+    blk_close<false>(tmem, &bars, T);
 }
 
 __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_adjoint_blk(LegArgs<float> a)
@@ -136,9 +135,8 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_leg_adjoint_blk(LegArgs<floa
     if (a.skip && *a.skip) return;
     const uint32_t tmem = blk_open(&s_tmem, &bars);
     const int m = blockIdx.x / a.blk_chunks;
-    uint32_t tiles = 0;
-    blk_adjoint_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tiles, tmem);
-    blk_close<true>(tmem, &bars, (int)tiles);
+    const int T = blk_adjoint_item(a, m, blockIdx.x - m * a.blk_chunks, blockIdx.y, smem, &bars, tmem);
+    blk_close<true>(tmem, &bars, T);
 }
 
 }  // namespace

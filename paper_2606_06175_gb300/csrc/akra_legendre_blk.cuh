@@ -318,12 +318,12 @@ __device__ __forceinline__ bool blk_wait(const LegArgs<float> &a, uint64_t *bar,
 // have no other waiter: waited for here by the thread that issued them, so that none is in flight when the block
 // gives its shared memory back (to a block that initialises barriers at the same addresses).
 template <bool ADJ>
-__device__ __forceinline__ bool blk_drain(const LegArgs<float> &a, BlkBars *bars, uint32_t end, int T, int h)
+__device__ __forceinline__ bool blk_drain(const LegArgs<float> &a, BlkBars *bars, int T, int h)
 {
     bool ok = true;
-    if (T > 0) ok &= blk_wait(a, &bars->bfree[(end - 1) & 1], (end - 1) >> 1);
-    if (T > 1) ok &= blk_wait(a, &bars->bfree[end & 1], (end - 2) >> 1);
-    if (ADJ && T > 0) ok &= blk_wait(a, &bars->yfree[h], end - 1);
+    if (T > 0) ok &= blk_wait(a, &bars->bfree[(T - 1) & 1], (T - 1) >> 1);
+    if (T > 1) ok &= blk_wait(a, &bars->bfree[T & 1], (T - 2) >> 1);
+    if (ADJ && T > 0) ok &= blk_wait(a, &bars->yfree[h], T - 1);
     return ok;
 }
 
@@ -356,10 +356,9 @@ struct BlkSynthSmem {
     static constexpr int BYTES = USED > 76 * 1024 ? USED : 76 * 1024;   // at most 2 blocks per SM (TMEM: 256 columns each)
 };
 
-// tiles: running count of the block's tiles (barrier phases)
-__device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const int m, const int chunk, const int r,
-                                               unsigned char *smem, BlkBars *bars, uint32_t &tiles,
-                                               const uint32_t tmem)
+// returns the number of tiles (uses of the barriers)
+__device__ __forceinline__ int blk_synth_item(const LegArgs<float> &a, const int m, const int chunk, const int r,
+                                              unsigned char *smem, BlkBars *bars, const uint32_t tmem)
 {
     using S = BlkSynthSmem;
     const int L = a.L;
@@ -392,7 +391,7 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
             BlkRaw nx;   // step tid of the next tile
             nx.load(a, m, mbase, lB + tid, r, lB + tid <= L);
             for (int t = 0; t < T; t++) {
-                const uint32_t gt = tiles + t;
+                const uint32_t gt = t;
                 const int buf = gt & 1, slot = gt & (BLK_SLOTS - 1);
                 float2 *s_cf = reinterpret_cast<float2 *>(smem + S::OFF_CF);
                 float4 *s_al = reinterpret_cast<float4 *>(smem + S::OFF_AL);
@@ -448,7 +447,7 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
             const uint32_t idesc = tc::idesc_f16(128, 64, 0, 0);
             const uint64_t vh = tc::sdesc_f16(va + h * 8192, 128, 512), vl = tc::sdesc_f16(va + h * 8192 + 256, 128, 512);
             for (int t = 0; t < T; t++) {
-                const uint32_t gt = tiles + t;
+                const uint32_t gt = t;
                 ok &= blk_wait(a, &bars->ready[gt & 1], gt >> 1);
 #pragma unroll
                 for (int u = 0; u < 2; u++) {   // half tile: 4 blocks
@@ -465,7 +464,7 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
                 }
                 tc::commit(&bars->bfree[gt & 1]);
             }
-            ok &= blk_drain<false>(a, bars, tiles + T, T, h);
+            ok &= blk_drain<false>(a, bars, T, h);
         }
     } else {
         float4 *s_al = reinterpret_cast<float4 *>(smem + S::OFF_PA);
@@ -525,7 +524,7 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
         blk_unscale(w[1]);
         const uint32_t col = tmem + ((uint32_t)(tid & 96) << 16);
         for (int t = 0; t < T; t++) {
-            const uint32_t gt = tiles + t;
+            const uint32_t gt = t;
             const float4 *ct = s_ct + (gt & (BLK_SLOTS - 1)) * BLK_NB;
 #pragma unroll
             for (int u = 0; u < 2; u++) {
@@ -566,8 +565,8 @@ __device__ __forceinline__ void blk_synth_item(const LegArgs<float> &a, const in
         }
     }
     if (!ok && a.err) atomicExch(a.err, 1);
-    tiles += T;
     __syncthreads();
+    return T;
 }
 
 // ---------------------------------------------------------------------------
@@ -594,9 +593,8 @@ struct BlkAdjSmem {
     static_assert(2 * (BYTES + 2048) <= 227 * 1024 && 3 * (BYTES + 1024) > 228 * 1024, "2 blocks per SM, whose TMEM fits");
 };
 
-__device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const int m, const int chunk, const int r,
-                                                 unsigned char *smem, BlkBars *bars, uint32_t &tiles,
-                                                 const uint32_t tmem)
+__device__ __forceinline__ int blk_adjoint_item(const LegArgs<float> &a, const int m, const int chunk, const int r,
+                                                unsigned char *smem, BlkBars *bars, const uint32_t tmem)
 {
     using S = BlkAdjSmem;
     const int L = a.L;
@@ -648,7 +646,7 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
         if (T > 0 && lB + tid <= L) pc = a.coef[AKRA_IX(mbase + lB + tid, ntri, kDbgCoef)];
         // the moments lag two tiles, so that a tile's jump values are there before the ring threads need them
         for (int t = 0; t < T + 2 && T > 0; t++) {
-            const uint32_t gt = tiles + t;
+            const uint32_t gt = t;
             if (t < T) {
                 const int buf = gt & 1, slot = gt & (BLK_SLOTS - 1);
                 float2 *s_cf = reinterpret_cast<float2 *>(smem + S::OFF_CF) + slot * S::ROWS;
@@ -772,7 +770,7 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
             const uint32_t id1 = tc::idesc_f16(128, 32, 0, 0), id2 = tc::idesc_f16(128, 32, 1, 1);
             const uint64_t vh = tc::sdesc_f16(va, 128, 512), vl = tc::sdesc_f16(va + 256, 128, 512);
             for (int t = 0; t <= T && T > 0; t++) {
-                const uint32_t gt = tiles + t, pt = gt - 1;
+                const uint32_t gt = t, pt = gt - 1;
                 if (t < T) {
                     ok &= blk_wait(a, &bars->ready[gt & 1], gt >> 1);
                     const uint32_t bb = tc::smem_u32(smem) + S::OFF_B + (gt & 1) * 2 * S::BBUF;
@@ -806,7 +804,7 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
                     tc::commit(&bars->full2[pt & 1]);
                 }
             }
-            ok &= blk_drain<true>(a, bars, tiles + T, T, h);
+            ok &= blk_drain<true>(a, bars, T, h);
         }
     } else {
 #pragma unroll
@@ -902,7 +900,7 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
         blk_bar_rings();   // phase A's buffers become the products'
         unsigned char *yrow = smem + S::OFF_Y + (tid >> 3) * 128 + (tid & 7) * 16;   // row tile k: + 2048 k
         for (int t = 0; t < T; t++) {
-            const uint32_t gt = tiles + t;
+            const uint32_t gt = t;
             const float2 *ct = s_ct + (gt & (BLK_SLOTS - 1)) * BLK_NB;
 #pragma unroll
             for (int u = 0; u < 2; u++) {
@@ -952,8 +950,8 @@ __device__ __forceinline__ void blk_adjoint_item(const LegArgs<float> &a, const 
         }
     }
     if (!ok && a.err) atomicExch(a.err, 1);
-    tiles += T;
     __syncthreads();
+    return T;
 }
 
 }  // namespace akra
