@@ -173,28 +173,28 @@ static bool jump_synth(akra_plan p, const LegShape &s, const int *units, int R)
 }
 
 // The adjoint's shape on a list of blk_pays: whether the block jumps take it (BA 2 or 0), for all of R, and the direct
-// shape where they do not.  The block jumps repeat for every right-hand side what a direct block does once (seeds, staging,
-// the warp reduction's set-up), compute the rings that pad a chunk, and pay a set-up, a slow first phase and a padded last
-// tile per block, for short l-ranges of many chunks above all.  Adjoint and epilogue in us, direct, block jumps (footprints:
-// DES-like; 30-degree cap):
-//   R = 1: 128 / 256 31, 24; 31, 26; 400 / 800 156, 158; 120, 124; 600 / 1200 376, 396; 288, 324; 1024 / 1024 399, 458; 349, 420; 2048 / 4096
-//          9857, 9172; 7316, 7465: the block jumps, whose errors are smaller by up to a third, but where lmax is below
-//          Nside (1500 / 1024 566, 668; 424, 558; 2048 / 1024 724, 878; 573, 749) and on a strip that fills its chunks badly (400 / 800,
-//          559 rings 125, 158)
-//   R = 2: 128 / 256 37, 35; 37, 35; 200 / 250 39, 45; 40, 36 (one chunk); 300 / 600 125, 143; 115, 140; 600 / 700 278, 323; 220, 260
-//   R = 5: 64 / 128 24, 30; 22, 30; 200 / 250 62, 92; 56, 63; 400 / 800 648, 743; 455, 566; 600 / 1200 1789, 1934; 1285, 1551
-//   R = 8: 400 / 400 296, 399; 221, 297; 1024 / 1024 3060, 3540; 2520, 3230; 1024 / 2048 11400, 11404; 9200, 10183
-// The direct shape is the one with the fewest pairs of padding: a single chunk up to 640 pairs, chunks of 384 or 512
-// beyond (400 / 800 with R = 5, 555 pairs: (5, 1) 648, (3, 1) 612, (4, 1) 728; 200 / 400, 278 pairs: (3, 1) 113, (2, 1) 139, (5, 1) 181).
+// shape where they do not.  The block jumps have the smaller errors (A^T by 1.1 to 1.6 times, growing with lmax), so they
+// stay wherever they are about as fast as the direct kernel they replaced at five pairs a thread.  They repeat for
+// every right-hand side what a direct block does once, compute the rings that pad a chunk, and pay a set-up, a slow first phase and
+// a padded last tile per block.  Whole A^T in us, that direct kernel, block jumps, this rule:
+//   lmax below Nside, many chunks: 1500 / 1024 cap 929, 1047, 910; 2048 / 1024 cap 1177, 1307, 1122, DES-like 1336, 1417, 1256
+//   several right-hand sides at low lmax (errors differ by a quarter at most there): 64 / 128 strip, R = 5 26, 36, 25; 128 / 256
+//          strip, R = 3 39, 45, 37; 200 / 250 DES-like, R = 5 154, 142, 112
+//   badly filled chunks: 400 / 800 strip R = 3 246, 325, 230, R = 8 632, 829, 536, R = 1 98, 119, 110 (a list that needs one
+//          side alone, for which the direct kernel does half the work); DES-like, 555 pairs in three chunks, R = 5 841, 884, 793
+//   the rest: DES-like, R = 5: 600 / 700 1291, 1225; 600 / 1200 2699, 2356; R = 1: 400 / 800 205, 191; 1024 / 1024 577, 579
+// (the strip: -0.45 < cos(theta) < 0).  The direct shape is the one with the fewest pairs of padding: a single chunk up to 640 pairs,
+// chunks of 384 or 512 beyond (adjoint alone, R = 5: 400 / 800, 555 pairs (5, 1) 648, (3, 1) 612, (4, 1) 728; 200 / 400, 278 pairs (3, 1) 113,
+// (2, 1) 139, (5, 1) 181).
 LegShape adjoint_shape(akra_plan p, const LegShape &s, const int *units, int nunits, int R)
 {
     LegShape t = s;
     if (s.BA != 1 || nunits <= 0 || !blk_pays(p, units, true)) return t;
     const BlkTables &bt = blk_tables(p, units);
-    const bool badly_filled = bt.nrows < 0.8 * 256 * bt.nchunks;
+    const bool badly_filled = bt.nrows < 0.8 * 256 * bt.nchunks && bt.nchunks >= (p->one_side ? 2 : R >= 3 ? 3 : kNeverLive);
     bool direct = bt.nchunks >= 3 && p->lmax < p->nside;
-    if (R >= 3 || (R == 2 && bt.nchunks >= 2)) direct |= p->lmax < 1100 || badly_filled;
-    if (R == 1 && bt.nchunks >= 2) direct |= badly_filled && p->one_side != 0 && p->nside * (double)p->lmax >= 2.2e5;
+    if (R >= 3 || (R == 2 && bt.nchunks >= 2)) direct |= p->lmax < 350 || badly_filled;
+    if (R == 1) direct |= badly_filled && p->nside * (double)p->lmax >= 2.2e5;
     t.BA = direct ? 0 : 2;
     if (!direct) return t;
     const int c = (nunits + 127) / 128;

@@ -20,32 +20,39 @@ def rel(a, b):
     return float((a.to(b.dtype) - b).norm() / b.norm())
 
 
-def _plan(N, L):
+ONE_SIDE, TWO_SIDES = (-0.95, -0.1), (-0.95, 0.02)   # cos(theta); the second needs both rings of a few pairs
+
+
+def _plan(N, L, sky=ONE_SIDE):
     z = np.cos(O.pixel_angles(N)[0])
     p = A.akra_plan_create(N, L)
-    A.akra_plan_set_weights(p, torch.from_numpy(np.where((z > -0.95) & (z < -0.1), 2.0, 0.0)).to(DEV), 1e-3)
+    A.akra_plan_set_weights(p, torch.from_numpy(np.where((z > sky[0]) & (z < sky[1]), 2.0, 0.0)).to(DEV), 1e-3)
     return p
 
 
 # adjoint of (Nside, lmax, R): the direct shape (ring pairs per thread, RHS per block), or None for the block jumps
 ROUTES = [
-    (64, 128, 2, None),           # one chunk of rings
-    (64, 128, 3, (1, 1)),         # 94 pairs
-    (400, 420, 1, None),          # one right-hand side
-    (200, 250, 2, (3, 1)),        # 293 pairs
-    (400, 420, 3, (5, 1)),        # 586 pairs: one chunk of 640
-    (300, 600, 4, (4, 1)),        # 439 pairs
-    (600, 500, 1, (4, 1)),        # lmax below Nside, four chunks, 878 pairs
-    (480, 479, 1, (3, 1)),        # 703 pairs: 768 slots in chunks of 384
-    (480, 480, 1, None),
-    (350, 1099, 3, (4, 1)),       # up to lmax 1100, 512 pairs
-    (350, 1100, 3, None),
+    (64, 128, 2, None, ONE_SIDE),         # one chunk of rings
+    (64, 128, 3, (1, 1), ONE_SIDE),       # 94 pairs
+    (200, 250, 2, (3, 1), ONE_SIDE),      # 293 pairs
+    (300, 349, 4, (4, 1), TWO_SIDES),     # up to lmax 350, 436 pairs
+    (300, 350, 4, None, TWO_SIDES),
+    (400, 420, 3, (5, 1), ONE_SIDE),      # 586 pairs that fill three chunks badly
+    (345, 420, 3, (5, 1), TWO_SIDES),     # 567 rings, 557 pairs, three chunks
+    (345, 420, 2, None, TWO_SIDES),
+    (120, 360, 3, None, ONE_SIDE),        # one chunk from lmax 350 on
+    (400, 420, 1, None, ONE_SIDE),
+    (400, 551, 1, (5, 1), ONE_SIDE),      # one right-hand side from Nside · lmax 220000 on
+    (300, 600, 4, None, ONE_SIDE),        # 439 pairs in two chunks that are not badly filled
+    (600, 500, 1, (4, 1), ONE_SIDE),      # lmax below Nside, four chunks, 878 pairs
+    (480, 479, 1, (3, 1), ONE_SIDE),      # 703 pairs: 768 slots in chunks of 384
+    (480, 480, 1, None, ONE_SIDE),
 ]
 
 
-@pytest.mark.parametrize("N,L,R,shape", ROUTES)
-def test_default_adjoint(N, L, R, shape):
-    p = _plan(N, L)
+@pytest.mark.parametrize("N,L,R,shape,sky", ROUTES)
+def test_default_adjoint(N, L, R, shape, sky):
+    p = _plan(N, L, sky)
     u = torch.randn(R, 2, 12 * N * N, device=DEV, generator=torch.Generator(device=DEV).manual_seed(N + L + R))
     b = A.akra_apply_At(p, A.F32, u, weighted=True)
     assert rel(b, A.akra_apply_At(p, A.F64, u.double(), weighted=True)) < tol32(L)
