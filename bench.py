@@ -72,15 +72,19 @@ def fp32_peak_tflops(sm_count, mhz):
     return sm_count * FP32_LANES * 2 * mhz * 1e6 / 1e12
 
 
-def kernel_source_sha():
-    """Short hash of the CUDA-core Legendre kernels' device code (scalar items and the paired
-    FP32 adjoint): a DRAM-traffic capture is only valid for the kernel code it was taken with.
-    Comments and blank lines are left out, so that an edit of the comments keeps a capture."""
+def kernel_source_sha(kernel=""):
+    """Short hash of a Legendre kernel's device code (the CUDA-core kernels' scalar items and paired
+    FP32 adjoint; for the block-jump kernels, k_leg_*_blk, also theirs): a DRAM-traffic capture
+    is only valid for the kernel code it was taken with.  Comments and blank lines are left out,
+    so that an edit of the comments keeps a capture."""
     import hashlib
     import re
 
     h = hashlib.sha256()
-    for f in ("akra_legendre_impl.cuh", "akra_legendre_f32x2.cuh"):
+    files = ["akra_legendre_impl.cuh", "akra_legendre_f32x2.cuh"]
+    if kernel.endswith("_blk"):
+        files += ["akra_legendre_blk.cuh", "akra_legendre_blk.cu", "akra_tc.cuh"]
+    for f in files:
         with open(os.path.join(ROOT, "paper_2606_06175_gb300", "csrc", f), encoding="utf-8") as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
@@ -96,7 +100,7 @@ def captured_traffic(kernel):
     dram_bytes_per_launch=<n>`).  (bytes, note); bytes is None when no capture matches the
     current kernel source."""
     path = os.path.join(PROFILES, "legendre_traffic_des2048.md")
-    sha = kernel_source_sha()
+    sha = kernel_source_sha(kernel)
     try:
         lines = open(path).read().splitlines()
     except OSError:
@@ -548,8 +552,9 @@ def main():
     peak = fp32_peak_tflops(sm_count, sm_max)
     work = legendre_flops(desc)
     dom = "legendre_adjoint" if st32["legendre_adjoint"] >= st32["legendre_synth"] else "legendre_synth"
-    # where nearly every ring pair needs one ring the block-jump kernels run (and few polar pairs' direct ones)
-    jump = work["steps_one_ring"] >= 0.9 * work["steps"]
+    # the library's rule for one RHS at lmax above Nside: where at least half of the steps are on ring pairs
+    # that need one ring the block-jump kernels run (and few polar pairs' direct ones)
+    jump = 2 * work["steps_one_ring"] >= work["steps"]
     kname = {"legendre_adjoint": "k_leg_adjoint", "legendre_synth": "k_leg_synth"}[dom] + ("_blk" if jump else "<float>")
     shape = A.akra_plan_get_shape(plan, A.F32, 1)
     rga = A.akra_plan_get_adjoint_shape(plan, A.F32, 1)["RGA"]

@@ -23,6 +23,17 @@
  *   - precision: AKRA_F64 -> double / complex double; AKRA_F32 -> float /
  *     complex float; AKRA_MIXED (cg_solve only) -> FP64 inputs and outputs, FP32 inner
  *     iterations, FP64 outer residual.
+ *     The FP32 operators (and FP32 inner iterations) are within 4 2^-24 lmax of FP64 in the
+ *     2-norm.  On footprints of one hemisphere (lmax >= 128), and for the synthesis over all
+ *     rings from lmax 4096 on, their Legendre stages may advance by blocks of 16 l-steps on the
+ *     tensor cores.  There the transfer polynomials, the interpolation weights and the adjoint's
+ *     products are held as two FP16 parts (22 bits; FP32 accumulation, the synthesis drops the
+ *     product of the two rests), the coefficients of 32 consecutive l and the maps' Fourier
+ *     coefficients of 256 rings share one power of two (a value below an eighth of the largest
+ *     has an absolute precision of 2^-25 of it), while the rings' cos theta enters in FP64.  The
+ *     error against FP64 is that of the direct FP32 recurrence or smaller (H at 512 / 1024 7.4e-6
+ *     against 9.3e-6, A^T at 1024 / 1024 9.5e-6 against 1.5e-5).  akra_plan_set_shape selects the
+ *     direct recurrence.
  *   - all array arguments named d_* are DEVICE pointers owned by the caller, 256-byte
  *     aligned as returned by cudaMalloc (or a torch CUDA tensor), contiguous.
  *   - stream: a cudaStream_t passed as void* (NULL = legacy default stream).  Calls are
@@ -247,7 +258,9 @@ akra_status akra_weight_grad(akra_plan plan, akra_prec prec, const void *d_Au, c
  * form is not in the paper.  Each FP32 H application of the inner CG runs as one persistent
  * Legendre-synthesis launch over the work items of all instances (a queue of
  * (instance, m, ring-pair chunk, RHS group) items, heaviest first), one ring-FFT launch over
- * all instances' rings and one persistent Legendre-adjoint launch. */
+ * all instances' rings and one persistent Legendre-adjoint launch.  Instances on footprints of one
+ * hemisphere (lmax >= 128) run block-jump Legendre launches of their own instead.  New weights of a
+ * member plan (akra_plan_set_weights) take effect with the next call. */
 typedef struct akra_batch_s *akra_batch;
 
 /* Group ninst plans (each with weights set; no plan twice) with R[i] RHS each (1..64).

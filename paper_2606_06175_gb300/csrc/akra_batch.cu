@@ -3,8 +3,9 @@
 // the work items of all instances (a queue of (instance, m, chunk, RHS group) items ordered
 // by cost, heaviest first), one ring-FFT launch over all instances' rings, one persistent
 // Legendre-adjoint launch, then each instance's epilogue and CG vector kernels -- all in one
-// CUDA graph per iteration.  The synthesis can instead run on the tensor cores (its own queue of
-// (instance, m, 128-pair chunk, RHS group) items; the adjoint keeps the CUDA-core items).  The FP64 outer refinement of the mixed-precision form runs per
+// CUDA graph per iteration.  Instances whose ring pairs the block-jump kernels take run those kernels'
+// launches instead of queue items.  The synthesis can instead run on the tensor cores (its own queue of
+// (instance, m, 128-pair chunk, RHS group) items; the adjoint stays as it is).  The FP64 outer refinement of the mixed-precision form runs per
 // instance between inner solves.  (Motivated by the paper's noise realisations and
 // tomographic bins, Sec. III; the batching itself is not in the paper.)
 #include <algorithm>

@@ -17,11 +17,12 @@
 //
 // Per (l, ring) step that needs one ring this leaves 16 tensor-core multiply-adds and about 2 FP32 ones where
 // the direct recurrence has 8 FP32 ones.  Measured on the DES-like footprint, one RHS, direct -> this:
-// Nside 2048 / lmax 4096 synthesis 8.19 -> 4.16 ms, adjoint 10.3 -> 8.8 ms; 512 / 1024 0.181 -> 0.125 ms,
-// 0.311 -> 0.223 ms.  What bounds it: no unit is busy half of the time (FMA pipe 38 %, tensor pipe 13 %,
-// shared memory 40 %); with TMEM for two blocks per SM a tile's way node threads -> product -> ring threads
-// -> freed columns (the product's round trip alone is 600 cycles) is not fully hidden, and about a fifth of
-// the time is phase A.
+// Nside 2048 / lmax 4096 synthesis 8.19 -> 4.16 ms, adjoint 10.3 (9.7 in its best shape) -> 8.8 ms; 512 / 1024 0.181 ->
+// 0.125 ms, 0.311 -> 0.223 ms.  Where they are not faster: akra_legendre.cu (jump_synth, adjoint_shape).  What
+// bounds it: no unit is busy half of the time (FMA pipe 43 % in the synthesis, 29 % in the adjoint, tensor pipe 15 and 9 %);
+// with TMEM for two blocks per SM a tile's way node threads -> product -> ring threads -> freed columns (the
+// product's round trip alone is 600 cycles) is not fully hidden, and phase A is more than a quarter of the time
+// (cycles a block at 2048 / 4096: synthesis 14.6k beside 13 tiles of 2.6k, adjoint 27.8k beside 13 of 4.8k).
 //
 // Precision: node values and V are split into two FP16 parts (22 bits), products head·head + head·rest +
 // rest·head with FP32 accumulation; nodes are FP32 numbers and V is computed in FP64 from the rings' FP64 x,
